@@ -7,7 +7,7 @@
 //   radix passes (per-tile digit histograms -> one prefix sum -> scatter; the
 //   first pass forms the Morton keys from the coordinates) -> finishing sort
 //   inside boxes + finest boxes -> coarser boxes -> child occupancy;
-// then for l = 2..L: job prefix -> list counts -> two prefix sums -> fill.
+// then per level l = 2..L two launches for the lists.
 // The host synchronises once at the end, and also: in cluster-size mode after
 // the sort (to learn each set's depth) and after the full-key sort of the sets
 // that need one; when the list capacity bound is too large, after the boxes.
@@ -466,7 +466,7 @@ struct Readback {
   DevStatus st{};
   std::vector<uint32_t> nbox;      // [nsets][kLevels] box counts
   std::vector<uint32_t> seg_long;  // [nsets]
-  std::vector<uint64_t> list;      // [kLevels][njobs][4]: base E2, base E4, nnz E2, nnz E4
+  std::vector<uint64_t> list;      // [kLevels][njobs][2]: E2 / E4 entries
   std::vector<uint32_t*> idx;      // [kLevels][2]: the level's E2 / E4 entry arrays
 };
 
@@ -1033,11 +1033,13 @@ int run_build(fmm_ctx* c, std::vector<SetPlan>& sets, std::vector<JobPlan>& jobs
     for (int l = 0; l <= sp.Lb; ++l) sp.cap[l] = level_cap(sp.n, l);
   }
 
-  // Zero-initialised words: every set's tickets, box counts and long-box
-  // flag side by side (one read-back copy for all sets), then per set its
-  // look-back words.
+  // Zero-initialised words: the list sizes, then every set's tickets, box
+  // counts and long-box flag side by side (one read-back copy for all of
+  // it), then per set its look-back words.
   constexpr size_t kSetWords = 2 + kLevels + 1;
-  size_t zero_bytes = align_up(sizeof(uint32_t) * kSetWords * nsets);
+  const size_t words_off = sizeof(uint64_t) * 2 * (size_t)njobs * kLevels;
+  const size_t read_bytes = words_off + sizeof(uint32_t) * kSetWords * nsets;
+  size_t zero_bytes = align_up(read_bytes);
   std::vector<size_t> zoff(nsets);
   for (uint32_t i = 0; i < nsets; ++i) {
     zoff[i] = zero_bytes;
@@ -1046,7 +1048,8 @@ int run_build(fmm_ctx* c, std::vector<SetPlan>& sets, std::vector<JobPlan>& jobs
   }
   char* zero = arena_get<char>(c, std::max<size_t>(zero_bytes, 1), &err);
   if (err) return err;
-  uint32_t* const set_words = reinterpret_cast<uint32_t*>(zero);
+  uint32_t* const set_words = reinterpret_cast<uint32_t*>(zero + words_off);
+  uint64_t* const nnz_words = reinterpret_cast<uint64_t*>(zero);
 
   // Per-set outputs.
   for (uint32_t i = 0; i < nsets; ++i) {
@@ -1137,7 +1140,7 @@ int run_build(fmm_ctx* c, std::vector<SetPlan>& sets, std::vector<JobPlan>& jobs
   };
 
   // List arrays (per level, shared by the jobs) and per-job row starts.
-  std::vector<size_t> work_len(kLevels, 0), zo_scan(kLevels, 0);
+  std::vector<uint32_t> chunks(kLevels, 0);
   char* list_zero = nullptr;
   size_t list_zero_bytes = 0;
   auto plan_lists = [&]() -> int {
@@ -1147,46 +1150,35 @@ int run_build(fmm_ctx* c, std::vector<SetPlan>& sets, std::vector<JobPlan>& jobs
       jp.dev.recv = jp.recv;
       jp.dev.L = jp.L;
     }
-    std::vector<size_t> zo(kLevels, 0), i2(kLevels, 0), i4(kLevels, 0);
+    std::vector<size_t> zo(kLevels, 0), room(kLevels, 0);
     for (int l = 2; l <= Lmax; ++l) {
-      size_t run = 0;
+      uint64_t parents = 0, rows = 0;
       for (auto& jp : jobs) {
         if (jp.L < l) continue;
-        jp.dev.region[l] = (uint32_t)run;
-        run += (size_t)jp.cap[l] + 1;
-        i2[l] += 27ull * jp.cap[l];
-        i4[l] += 189ull * jp.cap[l];
+        jp.dev.slot[l] = (uint32_t)room[l];
+        room[l] += ((size_t)jp.cap[l] + 3) & ~(size_t)3;
+        rows += (size_t)jp.cap[l] + 1;
+        parents += std::min<uint64_t>(jp.cap[l], sets[jp.recv].cap[l - 1]);
       }
-      if (run >= (1ull << 32)) return FMM_ERR_CAPACITY;
-      work_len[l] = run;
+      if (rows >= (1ull << 32) || room[l] >= (1ull << 32)) return FMM_ERR_CAPACITY;
+      chunks[l] = list_chunks(parents, njobs);
       zo[l] = list_zero_bytes;
-      // work arrays hold run + 1 entries: the scan writes its total at [run]
-      list_zero_bytes += 2 * align_up(sizeof(uint32_t) * (run + 1)) +
-                         2 * align_up(sizeof(uint64_t) * scan_tiles((uint32_t)run)) +
-                         align_up(sizeof(uint32_t) * 2) +
-                         2 * align_up(sizeof(uint64_t) * 2 * njobs) + align_up(sizeof(uint64_t) * 2);
+      list_zero_bytes += align_up(sizeof(uint32_t));
     }
     list_zero = arena_get<char>(c, std::max<size_t>(list_zero_bytes, 1), &err);
     if (err) return err;
     for (int l = 2; l <= Lmax; ++l) {
-      char* z = list_zero + zo[l];
-      const size_t run = work_len[l];
       ListLevel& LV = lvls[l];
-      LV.work2 = reinterpret_cast<uint32_t*>(z);
-      z += align_up(sizeof(uint32_t) * (run + 1));
-      LV.work4 = reinterpret_cast<uint32_t*>(z);
-      z += align_up(sizeof(uint32_t) * (run + 1));
-      zo_scan[l] = (size_t)(z - list_zero);
-      z += 2 * align_up(sizeof(uint64_t) * scan_tiles((uint32_t)run)) + align_up(sizeof(uint32_t) * 2);
-      LV.base = reinterpret_cast<uint64_t*>(z);
-      z += align_up(sizeof(uint64_t) * 2 * njobs);
-      LV.nnz = reinterpret_cast<uint64_t*>(z);
-      z += align_up(sizeof(uint64_t) * 2 * njobs);
-      LV.total = reinterpret_cast<uint64_t*>(z);
-      LV.idx2 = arena_get<uint32_t>(c, i2[l], &err);
-      LV.idx4 = arena_get<uint32_t>(c, i4[l], &err);
-      LV.code2 = l < Lmax ? arena_get<uint8_t>(c, i2[l], &err) : nullptr;
-      LV.jprefix = arena_get<uint32_t>(c, (size_t)njobs + 1, &err);
+      LV.ticket = reinterpret_cast<uint32_t*>(list_zero + zo[l]);
+      LV.nnz = nnz_words + (size_t)l * njobs * 2;
+      LV.off2 = arena_get<uint32_t>(c, 4ull * chunks[l], &err);
+      LV.off4 = arena_get<uint32_t>(c, 4ull * chunks[l], &err);
+      LV.bbase = arena_get<uint64_t>(c, 2ull * list_blocks() + 2ull * njobs, &err);
+      LV.jbase = LV.bbase + 2ull * list_blocks();
+      LV.idx2 = arena_get<uint32_t>(c, 27 * room[l], &err);
+      LV.idx4 = arena_get<uint32_t>(c, 189 * room[l], &err);
+      LV.code2 = l < Lmax ? arena_get<uint8_t>(c, 27 * room[l], &err) : nullptr;
+      LV.jchunks = arena_get<uint32_t>(c, (size_t)njobs + 1, &err);
       for (auto& jp : jobs) {
         if (jp.L < l) continue;
         jp.dev.out2[l] = arena_get<uint32_t>(c, (size_t)jp.cap[l] + 1, &err);
@@ -1247,27 +1239,18 @@ int run_build(fmm_ctx* c, std::vector<SetPlan>& sets, std::vector<JobPlan>& jobs
     launch_occupancy(m.segs, m.occ_slots, (uint32_t)occ.size(), m.occ_units, 0, c->st, s);
   }
 
-  auto read_sets = [&](bool lists) -> int {
-    const size_t list_words = lists ? 4 * (size_t)njobs * kLevels : 0;
-    const size_t need = 64 + sizeof(uint32_t) * nsets * kSetWords + 16 + sizeof(uint64_t) * list_words;
-    FMM_TRY(build_sync(c));  // the read-back buffer may be replaced
-    FMM_TRY(pinned_reserve(&c->rb_buf, &c->rb_bytes, need));
+  // Reads the status word, the box counts and the list sizes back in one copy.
+  auto read_sets = [&]() -> int {
+    if (64 + read_bytes > c->rb_bytes) {  // the read-back buffer is replaced
+      FMM_TRY(build_sync(c));
+      FMM_TRY(pinned_reserve(&c->rb_buf, &c->rb_bytes, 64 + read_bytes));
+    }
     char* h = static_cast<char*>(c->rb_buf);
     FMM_CUDA(cudaMemcpyAsync(h, c->st, sizeof(DevStatus), cudaMemcpyDeviceToHost, s));
-    uint32_t* hn = reinterpret_cast<uint32_t*>(h + 64);
-    FMM_CUDA(cudaMemcpyAsync(hn, set_words, sizeof(uint32_t) * nsets * kSetWords,
-                             cudaMemcpyDeviceToHost, s));
-    uint64_t* hl = reinterpret_cast<uint64_t*>(
-        (reinterpret_cast<uintptr_t>(hn + (size_t)nsets * kSetWords) + 15) & ~(uintptr_t)15);
-    if (lists)
-      for (int l = 2; l <= Lmax; ++l) {
-        FMM_CUDA(cudaMemcpyAsync(hl + (size_t)l * njobs * 4, lvls[l].base,
-                                 sizeof(uint64_t) * 2 * njobs, cudaMemcpyDeviceToHost, s));
-        FMM_CUDA(cudaMemcpyAsync(hl + (size_t)l * njobs * 4 + 2 * njobs, lvls[l].nnz,
-                                 sizeof(uint64_t) * 2 * njobs, cudaMemcpyDeviceToHost, s));
-      }
+    FMM_CUDA(cudaMemcpyAsync(h + 64, zero, read_bytes, cudaMemcpyDeviceToHost, s));
     FMM_TRY(build_sync(c));
     std::memcpy(&rb->st, h, sizeof(DevStatus));
+    const uint32_t* hn = reinterpret_cast<const uint32_t*>(h + 64 + words_off);
     rb->nbox.assign((size_t)nsets * kLevels, 0);
     rb->seg_long.assign(nsets, 0);
     for (uint32_t i = 0; i < nsets; ++i) {
@@ -1275,24 +1258,13 @@ int run_build(fmm_ctx* c, std::vector<SetPlan>& sets, std::vector<JobPlan>& jobs
                   sizeof(uint32_t) * kLevels);
       rb->seg_long[i] = hn[(size_t)i * kSetWords + 2 + kLevels];
     }
-    if (lists) {
-      rb->list.assign((size_t)kLevels * njobs * 4, 0);
-      for (int l = 2; l <= Lmax; ++l)
-        for (uint32_t j = 0; j < njobs; ++j) {
-          if (jobs[j].L < l) continue;
-          const uint64_t* b = hl + (size_t)l * njobs * 4;
-          uint64_t* o = &rb->list[((size_t)l * njobs + j) * 4];
-          o[0] = b[2 * j];
-          o[1] = b[2 * j + 1];
-          o[2] = b[2 * njobs + 2 * j];
-          o[3] = b[2 * njobs + 2 * j + 1];
-        }
-    }
+    const uint64_t* hl = reinterpret_cast<const uint64_t*>(h + 64);
+    rb->list.assign(hl, hl + (size_t)kLevels * njobs * 2);
     return FMM_OK;
   };
 
   if (!async_lists) {
-    FMM_TRY(read_sets(false));
+    FMM_TRY(read_sets());
     if (rb->st.code) return (int)rb->st.code;
     for (auto& jp : jobs)
       for (int l = 2; l <= jp.L; ++l) jp.cap[l] = rb->nbox[(size_t)jp.recv * kLevels + l];
@@ -1302,37 +1274,30 @@ int run_build(fmm_ctx* c, std::vector<SetPlan>& sets, std::vector<JobPlan>& jobs
   }
 
   // ---- lists, levels 2..Lmax.
+  if (njobs > 1 && Lmax >= 2) {
+    Launch Lk(c, "list_plan");
+    launch_list_plan(m.segs, m.jobs, njobs, Lmax, m.lvls, c->st, s);
+  }
   for (int l = 2; l <= Lmax; ++l) {
-    char* zs = list_zero + zo_scan[l];
-    const size_t sw = align_up(sizeof(uint64_t) * scan_tiles((uint32_t)work_len[l]));
-    uint64_t* st2 = reinterpret_cast<uint64_t*>(zs);
-    uint64_t* st4 = reinterpret_cast<uint64_t*>(zs + sw);
-    uint32_t* cnt = reinterpret_cast<uint32_t*>(zs + 2 * sw);
-    if (!job_prefix_in_count(njobs)) {
-      Launch Lk(c, "job_prefix");
-      launch_job_prefix(m.segs, m.jobs, njobs, l, m.lvls, c->st, s);
-    }
     {
       Launch Lk(c, "list_count");
-      launch_list_count(m.segs, m.jobs, njobs, l, m.lvls, c->st, s);
+      launch_list_count(m.segs, m.jobs, njobs, l, lvls[l], lvls[l - 1], chunks[l], c->st, s);
     }
-    {
-      Launch Lk(c, "scan");
-      launch_scan_u32_pair(lvls[l].work2, st2, lvls[l].total, lvls[l].work4, st4,
-                           lvls[l].total + 1, (uint32_t)work_len[l], cnt, c->st, wait_ns, s);
-    }
-    {
-      Launch Lk(c, "list_fill");
-      launch_list_fill(m.segs, m.jobs, njobs, l, m.lvls, lvls[l].code2 != nullptr, c->st, s);
-    }
+    Launch Lk(c, "list_fill");
+    launch_list_fill(m.segs, m.jobs, njobs, l, lvls[l], lvls[l - 1], chunks[l], c->st, s);
   }
   FMM_CUDA(cudaGetLastError());
 
   // ---- sizes and status.
-  FMM_TRY(read_sets(true));
+  FMM_TRY(read_sets());
   if (rb->st.code) return (int)rb->st.code;
   rb->idx.assign((size_t)kLevels * 2, nullptr);
   for (int l = 2; l <= Lmax; ++l) {
+    // (row starts are 32-bit; the bound holds over all jobs of a build)
+    uint64_t total[2] = {0, 0};
+    for (uint32_t j = 0; j < njobs; ++j)
+      for (int k = 0; k < 2; ++k) total[k] += rb->list[((size_t)l * njobs + j) * 2 + k];
+    if ((total[0] | total[1]) >> 32) return FMM_ERR_CAPACITY;
     rb->idx[2 * l] = lvls[l].idx2;
     rb->idx[2 * l + 1] = lvls[l].idx4;
   }
@@ -1401,13 +1366,13 @@ void fill_tree(const std::vector<SetPlan>& sets, const JobPlan& J, const Readbac
     }
   }
   for (int l = 2; l <= L; ++l) {
-    const uint64_t* o = &rb.list[((size_t)l * njobs + ji) * 4];
-    out->nnz_e2[l] = o[2];
-    out->nnz_e4[l] = o[3];
+    const uint64_t* o = &rb.list[((size_t)l * njobs + ji) * 2];
+    out->nnz_e2[l] = o[0];
+    out->nnz_e4[l] = o[1];
     out->e2_off[l] = J.dev.out2[l];
     out->e4_off[l] = J.dev.out4[l];
-    out->e2_idx[l] = rb.idx[2 * l] + o[0];
-    out->e4_idx[l] = rb.idx[2 * l + 1] + o[1];
+    out->e2_idx[l] = rb.idx[2 * l] + 27ull * J.dev.slot[l];
+    out->e4_idx[l] = rb.idx[2 * l + 1] + 189ull * J.dev.slot[l];
   }
 }
 
@@ -1837,7 +1802,7 @@ void workspace_parts(uint32_t N, uint32_t M, const fmm_params& p, uint64_t* byte
     for (int l = 0; l <= L; ++l) total += align_up(21ull * level_cap(ns[k], l) + 8) + 1024;
   }
   uint64_t lists = 0;
-  for (int l = 2; l <= L; ++l) lists += align_up(4ull * (4 + 27 + 189) * level_cap(M, l) + 64) + 4096;
+  for (int l = 2; l <= L; ++l) lists += align_up(4ull * (4 + 27 + 189) * level_cap(M, l) + 64) + 4096 + 16ull * list_blocks();
   *bytes = total;
   *list_bytes = lists;
 }

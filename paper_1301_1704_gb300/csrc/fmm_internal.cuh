@@ -342,31 +342,31 @@ __device__ __forceinline__ uint32_t find_slot(const Slot* slots, uint32_t nslots
 }
 
 // One (sources, receivers) pair whose E2 / E4 lists are built.  The list
-// arrays of a level are shared by all jobs of a build: counts go to the
-// job's region of the level's work array (scanned once for all jobs), list
-// entries to one array in job order; each job's row starts come out rebased
-// to its own lists.
+// arrays of a level are shared by all jobs of a build; a job's entries start
+// at a place the host fixes from the box-count bounds.
 struct Job {
   uint32_t src, recv;  // set indices
   int L;               // lists at levels 2..L
   uint32_t pad;
-  uint32_t region[kLevels];     // first entry of the job in the level's work array
-  uint32_t* out2[kLevels];      // rebased E2 row starts [nbox_recv + 1]
-  uint32_t* out4[kLevels];      // rebased E4 row starts
+  uint32_t slot[kLevels];       // receiver boxes the earlier jobs have room for (a multiple of 4):
+                                // the job's E2 entries start at 27 slot, its E4 entries at 189 slot
+  uint32_t* out2[kLevels];      // E2 row starts [nbox_recv + 1]
+  uint32_t* out4[kLevels];      // E4 row starts
 };
 
 // Per-level arrays shared by the jobs of a build.
 struct ListLevel {
-  uint32_t* work2;   // counts, then global row starts (all jobs)
-  uint32_t* work4;
   uint32_t* idx2;    // list entries (all jobs)
   uint32_t* idx4;
   uint8_t* code2;    // per E2 entry: (dx+1) + 3(dy+1) + 9(dz+1), the source box's offset
                      // from the receiver box; for the next level (null at the last one)
-  uint32_t* jprefix; // [njobs + 1] parents (receiver boxes at l-1) before each job
-  uint64_t* base;    // [njobs][2] first E2 / E4 entry of each job
-  uint64_t* nnz;     // [njobs][2] E2 / E4 entries of each job
-  uint64_t* total;   // [2] scanned totals of the level (capacity check)
+  uint32_t* jchunks; // [njobs + 1] chunks of four parents before each job (builds of several jobs)
+  uint32_t* off2;    // [4 chunks] a parent's first E2 / E4 entry, from its count block's first
+  uint32_t* off4;
+  uint64_t* bbase;   // [list_blocks()][2] first E2 / E4 entries of the count blocks
+  uint64_t* jbase;   // [njobs][2] ... and of the jobs
+  uint32_t* ticket;  // count blocks done (zeroed)
+  uint64_t* nnz;     // [njobs][2] E2 / E4 entries of each job (zeroed)
 };
 
 // One point set on the bucket path (bucket.cu): the points are bucketed on
@@ -524,25 +524,22 @@ uint32_t coarse_tiles(uint32_t cap);
 void launch_scan_u32(uint32_t* data, const uint32_t* count_dev, uint32_t cap, uint64_t* status,
                      uint32_t* counter, uint64_t* total64, DevStatus* st, uint64_t wait_ns,
                      cudaStream_t s);
-// The same for two arrays of cap entries each, in one launch.
-void launch_scan_u32_pair(uint32_t* data0, uint64_t* status0, uint64_t* total0, uint32_t* data1,
-                          uint64_t* status1, uint64_t* total1, uint32_t cap, uint32_t* counter,
-                          DevStatus* st, uint64_t wait_ns, cudaStream_t s);
 uint32_t scan_tiles(uint32_t cap);
 
-// Lists of level l for every job.  jprefix of the level is computed first
-// (parents before each job; 0 for jobs whose L < l).
-// lvls: device array of kLevels ListLevel (level l and its parent level l-1
-// are read).
-void launch_job_prefix(const Seg* segs, const Job* jobs, uint32_t njobs, int l,
-                       const ListLevel* lvls, DevStatus* st, cudaStream_t s);
-// Whether list_count computes the per-job prefix itself (small builds), so
-// that no job_prefix launch is needed.
-bool job_prefix_in_count(uint32_t njobs);
+// Lists of level l for every job, after one launch that plans the chunks of
+// every level (builds of several jobs; lvls: device array of kLevels
+// ListLevel).  lv, up: the host's copies of level l and of its parent level;
+// max_chunks: list_chunks of the level's parents.
+uint32_t list_chunks(uint64_t cap, uint32_t njobs);
+uint32_t list_blocks();
+void launch_list_plan(const Seg* segs, const Job* jobs, uint32_t njobs, int Lmax,
+                      const ListLevel* lvls, DevStatus* st, cudaStream_t s);
 void launch_list_count(const Seg* segs, const Job* jobs, uint32_t njobs, int l,
-                       const ListLevel* lvls, DevStatus* st, cudaStream_t s);
+                       const ListLevel& lv, const ListLevel& up, uint32_t max_chunks, DevStatus* st,
+                       cudaStream_t s);
 void launch_list_fill(const Seg* segs, const Job* jobs, uint32_t njobs, int l,
-                      const ListLevel* lvls, bool codes, DevStatus* st, cudaStream_t s);
+                      const ListLevel& lv, const ListLevel& up, uint32_t max_chunks, DevStatus* st,
+                      cudaStream_t s);
 
 // Bucket path (bucket.cu).  count and scatter: units = tiles of the slots'
 // sets (slot seg = BkSet index); plan: one block per set; split: units =

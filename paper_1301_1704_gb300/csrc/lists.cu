@@ -17,18 +17,27 @@
 // and walking Q in ascending rank, children in ascending octant, yields
 // ascending ranks.
 //
-// One warp handles one parent box p: lane k takes the k-th entry Q_k of
-// E2(p) (at most 27), and the warp serves every receiver child r of p.
-// Counting and filling are two kernels around a prefix sum of the counts.
+// Two launches a level.  The count kernel finds every parent's E2 and E4
+// entries and their prefix sums (of its receiver children together); the fill kernel
+// writes rows and entries, one warp a parent, no warp waiting for another.
+// Both walk the parents in chunks of four that never cross a job (a job's last
+// chunk may hold fewer): a warp takes a chunk at a time, so that the loads of
+// four parents are in flight together.
+#include <algorithm>
 #include <type_traits>
 
 #include "fmm_internal.cuh"
 
 namespace fmm {
 
-constexpr int kListWarps = kListThreads / 32;
-// Builds of at most this many jobs get their per-job prefix inside list_count.
-constexpr uint32_t kLocalJobs = 1024;
+constexpr int kChunk = 4;      // parents of a chunk
+constexpr int kNbor = 27;      // neighbours of a parent, at most
+constexpr int kCand = 27 * 8;  // candidates: the neighbours' children
+constexpr int kCountWarps = kListThreads / 32;
+constexpr int kCountPasses = 8;              // chunks a count warp takes in a row, at most
+constexpr uint32_t kCountGrid = 152u * 8u;   // eight blocks an SM
+constexpr int kFillWarps = kListThreads / 32;
+constexpr uint32_t kFillGrid = 152u * 4u;    // four blocks an SM
 
 __device__ __forceinline__ uint32_t axis_mask(int delta, uint32_t rho_bit, uint32_t lo_oct,
                                               uint32_t hi_oct) {
@@ -43,106 +52,124 @@ __device__ __forceinline__ uint32_t e2_child_mask(int dx, int dy, int dz, uint32
          axis_mask(dz, (rho >> 2) & 1u, 0x0fu, 0xf0u);
 }
 
-__device__ __forceinline__ uint32_t warp_sum(uint32_t v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
+// Population count of each byte.
+__device__ __forceinline__ uint32_t byte_popc(uint32_t v) {
+  v -= (v >> 1) & 0x55555555u;
+  v = (v & 0x33333333u) + ((v >> 2) & 0x33333333u);
+  return (v + (v >> 4)) & 0x0f0f0f0fu;
 }
 
-__device__ __forceinline__ uint32_t warp_excl(uint32_t v, int lane) {
-  uint32_t x = v;
+// Sum of the bytes of v (below 256 in all).
+__device__ __forceinline__ uint32_t byte_sum(uint32_t v) { return (v * 0x01010101u) >> 24; }
+
+// Bytes 0..3: all ones where bit 0..3 of m is set.
+__device__ __forceinline__ uint32_t byte_mask(uint32_t m) {
+  return (((m & 0xfu) * 0x00204081u) & 0x01010101u) * 0xffu;
+}
+
+// Inclusive prefix sum over the warp (the shuffle's own predicate says whether
+// the lane that far below exists).
+__device__ __forceinline__ uint32_t warp_incl(uint32_t x) {
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1)
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b32 y;\n\tshfl.sync.up.b32 y|p, %0, %1, 0, "
+        "0xffffffff;\n\t@p add.u32 %0, %0, y;\n\t}"
+        : "+r"(x)
+        : "r"(o));
+  return x;
+}
+
+__device__ __forceinline__ uint64_t warp_incl(uint64_t x) {
+  const int lane = threadIdx.x & 31;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+    const uint64_t y = __shfl_up_sync(0xffffffffu, x, o);
     if (lane >= o) x += y;
   }
-  return x - v;
+  return x;
 }
 
-// Everything one warp needs to serve the parents of one job at level l.
-struct ListCtx {
-  uint32_t nsrc1;              // non-empty source boxes at level 1 (level 2 only)
-  const uint64_t* rkey_up;     // receiver keys, level l-1
-  const uint32_t* rchild_up;   // receiver children, level l-1
-  const uint64_t* rkey;        // receiver keys, level l
-  const uint32_t* e2_off_up;   // the job's E2 row starts, level l-1 (rebased)
-  const uint32_t* e2_idx_up;   // the job's E2 entries, level l-1
-  const uint8_t* e2_code_up;   // ... and their offset codes (see list_fill), or null
-  const uint64_t* skey_up;     // source keys, level l-1
-  const uint32_t* schild_up;   // source children, level l-1
-  const uint8_t* socc_up;      // source child occupancy, level l-1
-  uint32_t region;             // the job's first entry in the level's work arrays
-  uint32_t nrecv;              // receiver boxes of the job at level l
-  uint32_t np;                 // parents (receiver boxes at l-1) of the job
-};
-
-__device__ __forceinline__ ListCtx make_ctx(const Seg* segs, const Job& J, int l,
-                                            const ListLevel* lvls, uint32_t jidx) {
-  const Seg& S = segs[J.src];
-  const Seg& R = segs[J.recv];
-  ListCtx c;
-  c.nsrc1 = S.nbox[1];
-  c.rkey_up = R.lv.key[l - 1];
-  c.rchild_up = R.lv.child[l - 1];
-  c.rkey = R.lv.key[l];
-  c.e2_off_up = l >= 3 ? J.out2[l - 1] : nullptr;
-  c.e2_idx_up = l >= 3 ? lvls[l - 1].idx2 + lvls[l - 1].base[2 * jidx] : nullptr;
-  c.e2_code_up = (l >= 3 && lvls[l - 1].code2) ? lvls[l - 1].code2 + lvls[l - 1].base[2 * jidx]
-                                               : nullptr;
-  c.skey_up = S.lv.key[l - 1];
-  c.schild_up = S.lv.child[l - 1];
-  c.socc_up = S.lv.occ[l - 1];
-  c.region = J.region[l];
-  c.nrecv = R.nbox[l];
-  c.np = 0;
-  return c;
+// Position of octant o among the 3 x 3 x 3 offsets: its part of an offset code.
+__host__ __device__ constexpr uint32_t oct_pos(uint32_t o) {
+  return (o & 1u) + 3u * ((o >> 1) & 1u) + 9u * (o >> 2);
 }
 
-// Per-lane view of one parent-level neighbour.
-struct Neighbour {
-  int dx, dy, dz;
-  uint32_t occ;
-  uint32_t child;
-};
+// Of a neighbour at offset code (dx+1) + 3(dy+1) + 9(dz+1): byte rho = its children
+// in sibling rho's E2.
+__device__ __forceinline__ uint2 code_masks(uint32_t code) {
+  const int dx = (int)(code % 3u) - 1, dy = (int)(code / 3u % 3u) - 1, dz = (int)(code / 9u) - 1;
+  uint32_t m[2] = {0, 0};
+  for (uint32_t rho = 0; rho < 8; ++rho)
+    m[rho >> 2] |= e2_child_mask(dx, dy, dz, rho) << (8 * (rho & 3));
+  return make_uint2(m[0], m[1]);
+}
 
-__device__ __forceinline__ Neighbour load_neighbour(const ListCtx& a, int l, uint32_t p, int lane) {
-  Neighbour q{0, 0, 0, 0u, 0u};
-  uint32_t m, first;
-  if (l == 2) {
-    first = 0;
-    m = a.nsrc1;
-  } else {
-    first = a.e2_off_up[p];
-    m = a.e2_off_up[p + 1] - first;
-  }
-  if ((uint32_t)lane < m) {
-    const uint32_t Q = (l == 2) ? (uint32_t)lane : a.e2_idx_up[first + lane];
-    if (a.e2_code_up) {
-      // the offset of Q from p, written with the entry: (dx+1) + 3(dy+1) + 9(dz+1)
-      const uint32_t code = a.e2_code_up[first + lane];
-      const uint32_t z = code / 9u, rem = code - 9u * z, y = rem / 3u;
-      q.dx = (int)(rem - 3u * y) - 1;
-      q.dy = (int)y - 1;
-      q.dz = (int)z - 1;
-    } else {
-      const uint64_t pk = a.rkey_up[p];
-      const uint64_t qk = a.skey_up[Q];
-      q.dx = (int)compact3(qk) - (int)compact3(pk);
-      q.dy = (int)compact3(qk >> 1) - (int)compact3(pk >> 1);
-      q.dz = (int)compact3(qk >> 2) - (int)compact3(pk >> 2);
+// Chunks a count warp takes in a row in a level of `chunks`: small levels are
+// spread over the SMs, one chunk a warp.
+__host__ __device__ inline uint32_t count_passes(uint32_t chunks) {
+  const uint32_t p = chunks / (kCountGrid * kCountWarps);
+  return p < 1u ? 1u : (p > (uint32_t)kCountPasses ? (uint32_t)kCountPasses : p);
+}
+
+// Chunks of a count block: whole tiles of its warps' passes, one range a block.
+__device__ __forceinline__ uint32_t count_range(uint32_t chunks) {
+  const uint32_t tile = count_passes(chunks) * kCountWarps;
+  const uint32_t tiles = (chunks + tile - 1) / tile;
+  return tile * ((tiles + kCountGrid - 1) / kCountGrid);
+}
+
+// Chunks of a job with np parents at level l.
+__device__ __forceinline__ uint32_t job_chunks(const Job& J, const Seg* segs, int l) {
+  return J.L < l ? 0u : (segs[J.recv].nbox[l - 1] + kChunk - 1) / kChunk;
+}
+
+// Chunks of a level of at most `cap` parents in all, at most.
+uint32_t list_chunks(uint64_t cap, uint32_t njobs) { return (uint32_t)(cap / kChunk) + njobs; }
+uint32_t list_blocks() { return kCountGrid; }
+
+// Per level (one block each): the chunks before each job.
+__global__ void __launch_bounds__(1024) list_plan_kernel(const Seg* __restrict__ segs,
+                                                         const Job* __restrict__ jobs,
+                                                         uint32_t njobs, const ListLevel* lvls,
+                                                         const DevStatus* st) {
+  __shared__ uint32_t s_sum[33];
+  if (failed(st)) return;
+  const int l = 2 + blockIdx.x;
+  const ListLevel& LV = lvls[l];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint32_t before = 0;
+  for (uint32_t c = 0; c < njobs; c += blockDim.x) {
+    const uint32_t j = c + threadIdx.x;
+    const uint32_t v = j < njobs ? job_chunks(jobs[j], segs, l) : 0u;
+    const uint32_t x = warp_incl(v);
+    __syncthreads();
+    if (lane == 31) s_sum[warp] = x;
+    __syncthreads();
+    if (warp == 0) {
+      const uint32_t w = s_sum[lane], y = warp_incl(w);
+      s_sum[lane] = y - w;
+      if (lane == 31) s_sum[32] = y;
     }
-    q.occ = a.socc_up[Q];
-    q.child = a.schild_up[Q];
+    __syncthreads();
+    if (j < njobs) LV.jchunks[j] = before + s_sum[warp] + x - v;
+    before += s_sum[32];
   }
-  return q;
+  if (threadIdx.x == 0) LV.jchunks[njobs] = before;
 }
 
-// Job holding global parent g: jp[j] <= g < jp[j + 1].
-__device__ __forceinline__ uint32_t find_job(const uint32_t* jp, uint32_t njobs, uint32_t g) {
+void launch_list_plan(const Seg* segs, const Job* jobs, uint32_t njobs, int Lmax,
+                      const ListLevel* lvls, DevStatus* st, cudaStream_t s) {
+  if (njobs <= 1 || Lmax < 2) return;  // one job: its chunks follow from its box counts
+  list_plan_kernel<<<(uint32_t)(Lmax - 1), 1024, 0, s>>>(segs, jobs, njobs, lvls, st);
+}
+
+// Job whose chunks hold chunk c: jc[j] <= c < jc[j + 1].
+__device__ __forceinline__ uint32_t find_job(const uint32_t* jc, uint32_t njobs, uint32_t c) {
   uint32_t lo = 0, hi = njobs;
   while (hi - lo > 1) {
     const uint32_t mid = (lo + hi) >> 1;
-    if (jp[mid] <= g)
+    if (jc[mid] <= c)
       lo = mid;
     else
       hi = mid;
@@ -150,467 +177,611 @@ __device__ __forceinline__ uint32_t find_job(const uint32_t* jp, uint32_t njobs,
   return lo;
 }
 
-// Parents before each job at level l (0 for jobs whose lists stop below l).
-__global__ void job_prefix_kernel(const Seg* __restrict__ segs, const Job* __restrict__ jobs,
-                                  uint32_t njobs, int l, const ListLevel* lvls, DevStatus* st) {
-  __shared__ uint32_t s_carry, s_wsum[32];
-  if (failed(st)) return;
-  const ListLevel& LV = lvls[l];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int nw = blockDim.x >> 5;
-  if (threadIdx.x == 0) s_carry = 0;
-  __syncthreads();
-  for (uint32_t c = 0; c < njobs; c += blockDim.x) {
-    const uint32_t j = c + threadIdx.x;
-    uint32_t np = 0;
-    if (j < njobs && jobs[j].L >= l) {
-      const Seg& R = segs[jobs[j].recv];
-      np = R.nbox[l - 1];
-      if (R.nbox[l] == 0) {
-        jobs[j].out2[l][0] = 0;
-        jobs[j].out4[l][0] = 0;
-      }
-    }
-    uint32_t x = np;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-      if (lane >= o) x += y;
-    }
-    if (lane == 31) s_wsum[warp] = x;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      uint32_t run = s_carry;
-      for (int w = 0; w < nw; ++w) {
-        const uint32_t v = s_wsum[w];
-        s_wsum[w] = run;
-        run += v;
-      }
-      s_carry = run;
-    }
-    __syncthreads();
-    if (j < njobs) LV.jprefix[j] = s_wsum[warp] + x - np;
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) LV.jprefix[njobs] = s_carry;
-}
-
-void launch_job_prefix(const Seg* segs, const Job* jobs, uint32_t njobs, int l,
-                       const ListLevel* lvls, DevStatus* st, cudaStream_t s) {
-  job_prefix_kernel<<<1, 1024, 0, s>>>(segs, jobs, njobs, l, lvls, st);
-}
-
-bool job_prefix_in_count(uint32_t njobs) { return njobs <= kLocalJobs; }
-
-// Each block takes a contiguous run of the level's parents (over all jobs),
-// dealt round-robin to its warps: a warp changes jobs only where the run
-// crosses a job boundary, and the warps of a block work on neighbouring
-// parents, whose list stores land close together.
-struct BlockRange {
-  uint32_t g0, g1;
+// A warp's current job at level l.
+struct WarpJob {
+  const uint32_t* off_up;   // E2 row starts, level l-1
+  const uint32_t* idx_up;   // E2 entries, level l-1
+  const uint8_t* code_up;   // ... and their offset codes
+  const uint32_t* rchild;   // receiver children, level l-1
+  const uint64_t* rkey;     // receiver keys, level l
+  const uint8_t* socc;      // source child occupancy, level l-1
+  const uint32_t* schild;   // source children, level l-1
+  uint32_t* out2;           // row starts, level l
+  uint32_t* out4;
+  uint64_t base2, base4;    // the level's entries before the job
+  uint32_t j, chunk0, chunk1, np, nsrc1;
+  uint64_t slot;
 };
 
-__device__ __forceinline__ BlockRange block_range(uint32_t total) {
-  const uint32_t per = (uint32_t)(((uint64_t)total + gridDim.x - 1) / gridDim.x);
-  const uint64_t a = (uint64_t)blockIdx.x * per, b = a + per;
-  return BlockRange{(uint32_t)(a < total ? a : total), (uint32_t)(b < total ? b : total)};
+__device__ void load_job(WarpJob& W, const Seg* segs, const Job* jobs, uint32_t njobs, int l,
+                         const ListLevel& LV, const ListLevel& up, uint32_t c) {
+  const uint32_t j = njobs == 1 ? 0u : find_job(LV.jchunks, njobs, c);
+  const Job& J = jobs[j];
+  const Seg& S = segs[J.src];
+  const Seg& R = segs[J.recv];
+  W.j = j;
+  W.np = R.nbox[l - 1];
+  W.chunk0 = njobs == 1 ? 0u : LV.jchunks[j];
+  W.chunk1 = njobs == 1 ? (W.np + kChunk - 1) / kChunk : LV.jchunks[j + 1];
+  W.nsrc1 = min(S.nbox[1], 8u);
+  W.off_up = J.out2[l - 1];
+  W.idx_up = l > 2 ? up.idx2 + 27ull * J.slot[l - 1] : nullptr;
+  W.code_up = l > 2 ? up.code2 + 27ull * J.slot[l - 1] : nullptr;
+  W.rchild = R.lv.child[l - 1];
+  W.rkey = R.lv.key[l];
+  W.socc = S.lv.occ[l - 1];
+  W.schild = S.lv.child[l - 1];
+  W.out2 = J.out2[l];
+  W.out4 = J.out4[l];
+  W.slot = J.slot[l];
 }
 
-// Parents before each job at level l, computed by the whole block into s_jp
-// (njobs <= kLocalJobs; s_jp[kLocalJobs] = the level's total).  Block 0 also
-// publishes them in `jprefix_out` for the fill kernel and starts the rows of
-// jobs with no receiver box at level l, as job_prefix_kernel does for larger
-// builds.
-
-__device__ void block_job_prefix(const Seg* __restrict__ segs, const Job* __restrict__ jobs,
-                                 uint32_t njobs, int l, uint32_t* s_jp, uint32_t* s_wsum,
-                                 uint32_t* jprefix_out) {
-  constexpr int kPer = kLocalJobs / kListThreads;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  uint32_t v[kPer], sum = 0;
-#pragma unroll
-  for (int k = 0; k < kPer; ++k) {
-    const uint32_t j = threadIdx.x * kPer + k;
-    v[k] = 0;
-    if (j < njobs && jobs[j].L >= l) {
-      const Seg& R = segs[jobs[j].recv];
-      v[k] = R.nbox[l - 1];
-      if (blockIdx.x == 0 && R.nbox[l] == 0) {
-        jobs[j].out2[l][0] = 0;
-        jobs[j].out4[l][0] = 0;
-      }
-    }
-    sum += v[k];
-  }
-  uint32_t x = sum;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) s_wsum[warp] = x;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    uint32_t run = 0;
-    for (int w = 0; w < kListWarps; ++w) {
-      const uint32_t c = s_wsum[w];
-      s_wsum[w] = run;
-      run += c;
-    }
-    s_jp[kLocalJobs] = run;
-  }
-  __syncthreads();
-  uint32_t off = s_wsum[warp] + x - sum;
-#pragma unroll
-  for (int k = 0; k < kPer; ++k) {
-    s_jp[threadIdx.x * kPer + k] = off;
-    off += v[k];
-  }
-  __syncthreads();
-  if (blockIdx.x == 0)
-    for (uint32_t j = threadIdx.x; j <= njobs; j += blockDim.x)
-      jprefix_out[j] = j < kLocalJobs ? s_jp[j] : s_jp[kLocalJobs];
+// At level 2 every pair of level-1 boxes touches: the offset code follows from
+// their octants.
+__device__ __forceinline__ uint32_t level1_code(uint32_t source, uint32_t receiver) {
+  return 13u + oct_pos(source) - oct_pos(receiver);
 }
 
 // Counts: per receiver child r of parent p, |E2(r)| = sum over the parent's
 // neighbours Q of popc(occ(Q) & mask(delta_Q, rho_r)), and |E2| + |E4| = the
-// number of non-empty children of all Q.  The eight possible sibling octants
-// are counted at once: byte rho of a packed pair of words.  The kernel waits
-// on chains of dependent loads (row start, entry, occupancy): eight blocks an
-// SM keep more parents in flight.
-__global__ void __launch_bounds__(kListThreads, 8) list_count_kernel(const Seg* __restrict__ segs,
-                                                                 const Job* __restrict__ jobs,
-                                                                 uint32_t njobs, int l,
-                                                                 const ListLevel* lvls,
-                                                                 DevStatus* st) {
-  __shared__ uint32_t s_jp[kLocalJobs + 1];
-  __shared__ uint32_t s_wsum[kListWarps];
+// number of non-empty children of all Q.  Eight lanes a parent, four parents a
+// warp pass; the eight sibling octants are counted at once, as bytes.  The
+// kernel waits on chains of dependent loads (row start, entry, occupancy), so
+// it keeps many warps in flight.  off2 / off4: a parent's first entries, from
+// the block's first; the last block to finish turns the blocks' totals
+// into their prefix sums and closes the jobs' rows.  Offsets a parent, not a
+// receiver box, and no separate prefix sum over them: 116 us for levels 2..7
+// of 2^24 uniform points, against 187 us for a warp a parent, counts a receiver
+// box and a prefix sum launch a level.
+__global__ void __launch_bounds__(kListThreads, 6) list_count_kernel(
+    const Seg* __restrict__ segs, const Job* __restrict__ jobs, uint32_t njobs, int l,
+    const __grid_constant__ ListLevel LV, const __grid_constant__ ListLevel up, DevStatus* st) {
+  __shared__ uint2 s_mask[kNbor];
+  __shared__ WarpJob s_job[kCountWarps];
+  __shared__ uint64_t s_sum[2][kCountWarps + 1];
+  __shared__ uint32_t s_last;
   if (failed(st)) return;  // set before this launch: the same for every thread
-  const int lane = threadIdx.x & 31;
-  // The level's arrays in registers: stores through them must not force
-  // reloads of the descriptor.
-  uint32_t* const work2 = lvls[l].work2;
-  uint32_t* const work4 = lvls[l].work4;
-  const uint32_t* jprefix = lvls[l].jprefix;
-  if (njobs <= kLocalJobs) {  // the per-job prefix here, not in its own launch
-    block_job_prefix(segs, jobs, njobs, l, s_jp, s_wsum, lvls[l].jprefix);
-    jprefix = s_jp;
-  }
-  const uint32_t total = njobs <= kLocalJobs ? s_jp[kLocalJobs] : jprefix[njobs];
-  const BlockRange br = block_range(total);
-  uint32_t j = 0, jstart = 0, jend = 0;
-  ListCtx a{};
-  for (uint32_t g = br.g0 + (threadIdx.x >> 5); g < br.g1; g += blockDim.x >> 5) {
-    if (g >= jend) {  // g only grows: look its job up when it leaves the current one
-      j = find_job(jprefix, njobs, g);
-      a = make_ctx(segs, jobs[j], l, lvls, j);
-      jstart = jprefix[j];
-      jend = jprefix[j + 1];
-    }
-    const uint32_t p = g - jstart;
-    const Neighbour q = load_neighbour(a, l, p, lane);
-    uint32_t lo = 0, hi = 0;  // byte rho: popc(occ & mask(delta, rho))
-    {
-      // mask(delta, rho) factors by axis into masks chosen by rho's bits
-      const uint32_t mx0 = axis_mask(q.dx, 0u, 0x55u, 0xaau), mx1 = axis_mask(q.dx, 1u, 0x55u, 0xaau);
-      const uint32_t my0 = axis_mask(q.dy, 0u, 0x33u, 0xccu), my1 = axis_mask(q.dy, 1u, 0x33u, 0xccu);
-      const uint32_t mz0 = axis_mask(q.dz, 0u, 0x0fu, 0xf0u), mz1 = axis_mask(q.dz, 1u, 0x0fu, 0xf0u);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int sub = lane >> 3, l8 = lane & 7;
+  const uint32_t chunks = njobs == 1 ? job_chunks(jobs[0], segs, l) : LV.jchunks[njobs];
+  const uint32_t passes = count_passes(chunks), range = count_range(chunks);
+  const uint32_t b0 = blockIdx.x * range;
+  const uint32_t nblocks = range ? (chunks + range - 1) / range : 0u;
+  if (blockIdx.x >= max(nblocks, 1u)) return;
+  if (tid < kNbor) s_mask[tid] = code_masks(tid);
+  __syncthreads();
+  WarpJob& W = s_job[warp];
+  uint32_t jend = 0;
+  uint64_t run2 = 0, run4 = 0;  // the block's entries so far
+  const uint32_t b1 = min(b0 + range, chunks);
+  for (uint32_t t0 = b0; t0 < b1; t0 += passes * kCountWarps) {
+    const uint32_t c0 = t0 + warp * passes;
+    uint32_t keep2 = 0, keep4 = 0;  // lane 4 k + i: parent i of the warp's chunk k
+    for (uint32_t k = 0; k < passes; ++k) {
+      const uint32_t c = c0 + k;
+      uint32_t n2 = 0, n4 = 0;
+      if (c < b1) {
+        if (c >= jend) {  // c only grows
+          __syncwarp();
+          if (lane == 0) load_job(W, segs, jobs, njobs, l, LV, up, c);
+          __syncwarp();
+          jend = W.chunk1;
+        }
+        const uint32_t p = (c - W.chunk0) * kChunk + sub;
+        const bool in = p < W.np;
+        uint32_t first = 0, m = 0, r0 = 0, nch = 0;
+        if (in) {
+          r0 = W.rchild[p];
+          nch = min(W.rchild[p + 1] - r0, 8u);
+          if (l == 2) {
+            m = W.nsrc1;
+          } else {
+            first = W.off_up[p];
+            m = min(W.off_up[p + 1] - first, (uint32_t)kNbor);
+          }
+        }
+        uint32_t q[4], code[4];
 #pragma unroll
-      for (uint32_t rho = 0; rho < 8; ++rho) {
-        const uint32_t m = ((rho & 1) ? mx1 : mx0) & ((rho & 2) ? my1 : my0) & ((rho & 4) ? mz1 : mz0);
-        const uint32_t cnt = (uint32_t)__popc(q.occ & m);
-        if (rho < 4)
-          lo |= cnt << (8 * rho);
-        else
-          hi |= cnt << (8 * (rho - 4));
+        for (int u = 0; u < 4; ++u) {
+          const uint32_t i = l8 + 8 * u;
+          q[u] = i;
+          code[u] = 13;
+          if (i < m) {
+            if (l == 2) {
+              code[u] = level1_code((uint32_t)segs[jobs[W.j].src].lv.key[1][i],
+                                    (uint32_t)segs[jobs[W.j].recv].lv.key[1][p]);
+            } else {
+              q[u] = W.idx_up[first + i];
+              code[u] = W.code_up[first + i];
+            }
+          }
+        }
+        const uint32_t oct = (uint32_t)l8 < nch ? 1u << (uint32_t)(W.rkey[r0 + l8] & 7u) : 0u;
+        uint32_t lo = 0, hi = 0, tp = oct << 16;  // tp: candidates | octants of the children << 16
+        uint32_t occ[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) occ[u] = (uint32_t)l8 + 8 * u < m ? W.socc[q[u]] : 0u;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const uint2 mk = s_mask[code[u]];
+          const uint32_t occ4 = occ[u] * 0x01010101u;
+          lo += byte_popc(mk.x & occ4);
+          hi += byte_popc(mk.y & occ4);
+          tp += __popc(occ[u]);
+        }
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) {
+          lo += __shfl_xor_sync(0xffffffffu, lo, o);
+          hi += __shfl_xor_sync(0xffffffffu, hi, o);
+          tp += __shfl_xor_sync(0xffffffffu, tp, o);
+        }
+        const uint32_t present = tp >> 16;
+        n2 = byte_sum(lo & byte_mask(present)) + byte_sum(hi & byte_mask(present >> 4));
+        n4 = (uint32_t)__popc(present) * (tp & 0xffffu) - n2;
+      }
+      // lane 4 k + i takes parent i's counts (its group: lanes 8 i ..)
+      const uint32_t v2 = __shfl_sync(0xffffffffu, n2, (lane & 3) * 8);
+      const uint32_t v4 = __shfl_sync(0xffffffffu, n4, (lane & 3) * 8);
+      if ((uint32_t)(lane >> 2) == k) {
+        keep2 = v2;
+        keep4 = v4;
       }
     }
-    const uint32_t tot = warp_sum(__popc(q.occ));
-    lo = warp_sum(lo);
-    hi = warp_sum(hi);
-    const uint32_t c0 = a.rchild_up[p];
-    const uint32_t c1 = min(a.rchild_up[p + 1], c0 + 8u);  // (at most 8 in a whole tree)
-    const uint32_t r = c0 + lane;
-    if (r < c1) {
-      const uint32_t rho = (uint32_t)(a.rkey[r] & 7u);
-      const uint32_t n2 = ((rho < 4 ? lo : hi) >> (8 * (rho & 3))) & 0xffu;
-      work2[a.region + r] = n2;
-      work4[a.region + r] = tot - n2;
+    const uint32_t x2 = warp_incl(keep2), x4 = warp_incl(keep4);
+    if (lane == 31) {
+      s_sum[0][warp] = x2;
+      s_sum[1][warp] = x4;
+    }
+    __syncthreads();
+    uint64_t w2 = run2, w4 = run4;
+#pragma unroll
+    for (int w = 0; w < kCountWarps; ++w) {
+      const uint64_t a = s_sum[0][w], b = s_sum[1][w];
+      if (w < warp) {
+        w2 += a;
+        w4 += b;
+      }
+      run2 += a;
+      run4 += b;
+    }
+    __syncthreads();
+    const uint32_t c = c0 + (lane >> 2);
+    if ((uint32_t)(lane >> 2) < passes && c < b1) {
+      LV.off2[(uint64_t)c * kChunk + (lane & 3)] = (uint32_t)w2 + x2 - keep2;
+      LV.off4[(uint64_t)c * kChunk + (lane & 3)] = (uint32_t)w4 + x4 - keep4;
+    }
+  }
+  if (tid == 0) {
+    LV.bbase[2 * blockIdx.x] = run2;
+    LV.bbase[2 * blockIdx.x + 1] = run4;
+  }
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) s_last = atomicAdd(LV.ticket, 1u) + 1u == max(nblocks, 1u);
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+
+  // The last block: the blocks' first entries, then per job its first entry,
+  // its totals and its closing rows.  (Reads past L1: other blocks wrote them.)
+  constexpr int kPer = (kCountGrid + kListThreads - 1) / kListThreads;
+  uint64_t tot[2] = {0, 0};
+#pragma unroll
+  for (int d = 0; d < 2; ++d) {
+    uint64_t v[kPer], sum = 0;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      const uint32_t b = tid * kPer + k;
+      v[k] = b < nblocks ? __ldcg(LV.bbase + 2 * b + d) : 0ull;
+      sum += v[k];
+    }
+    const uint64_t x = warp_incl(sum);
+    if (lane == 31) s_sum[d][warp] = x;
+    __syncthreads();
+    uint64_t e = x - sum;
+    for (int w = 0; w < kCountWarps; ++w) {
+      if (w < warp) e += s_sum[d][w];
+      tot[d] += s_sum[d][w];
+    }
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      const uint32_t b = tid * kPer + k;
+      if (b < nblocks) LV.bbase[2 * b + d] = e;
+      e += v[k];
+    }
+    __syncthreads();
+  }
+  for (uint32_t j = tid; j < njobs; j += kListThreads) {
+    const Job& J = jobs[j];
+    if (J.L < l) continue;
+    const uint32_t ca = njobs == 1 ? 0u : LV.jchunks[j];
+    const uint32_t cb = njobs == 1 ? chunks : LV.jchunks[j + 1];
+    const auto entry = [&](uint32_t c, int d) -> uint64_t {
+      if (c >= chunks) return tot[d];
+      return LV.bbase[2 * (c / range) + d] + __ldcg((d ? LV.off4 : LV.off2) + (uint64_t)c * kChunk);
+    };
+    const uint32_t nrecv = segs[J.recv].nbox[l];
+    for (int d = 0; d < 2; ++d) {
+      const uint64_t a = entry(ca, d), n = entry(cb, d) - a;
+      LV.jbase[2 * j + d] = a;
+      LV.nnz[2 * j + d] = n;
+      (d ? J.out4[l] : J.out2[l])[nrecv] = (uint32_t)n;
+      if (n >> 32) set_error(st, FMM_ERR_CAPACITY);
     }
   }
 }
 
-// Fill: per parent p, the candidate list C -- the non-empty children of p's
-// neighbours in ascending rank -- is built once in shared memory with, per
-// candidate, the byte of sibling octants rho whose E2 it belongs to.  Because
-// the E2 condition |2 delta + o - rho| <= 1 is symmetric under
-// (delta, o, rho) -> (-delta, rho, o), that byte is e2_child_mask(-delta, o).
-// Every receiver child then splits C by one ballot per 32 candidates: its E2
-// and E4 lists come out in ascending order as contiguous, coalesced stores.
-// Row starts are written rebased to the job's own lists.
-constexpr int kCand = 27 * 8;  // at most 27 neighbours x 8 children
-constexpr int kNear = 64;      // candidates in some sibling's E2: the 4x4x4 block
-constexpr uint32_t kStage = 4 * 189 + 4;  // four E4 lists, and up to 3 entries of alignment
-constexpr uint32_t kStageMin = 128;       // candidates of a parent whose E4 lists are staged
-constexpr uint32_t kStageJob = 1u << 25;  // E4 entries of a job's level whose lists are staged
-
-// A warp's current job in the fill kernel.
-struct WarpJob {
-  ListCtx a;
-  uint32_t* out2;  // the job's row starts, level l
-  uint32_t* out4;
-  uint32_t G2, G4;  // the job's first entries in the level's lists
-  uint32_t j, jstart, jend;
-  uint32_t big;     // the job's E4 lists at this level outgrow L2
-};
-
+// Fill.  Per parent p, the candidate list C -- the non-empty children of p's
+// neighbours in ascending rank -- is built in shared memory.  p's receiver
+// children, its siblings, are numbered 0..nsib-1 in order.  Every candidate
+// carries its rank, a flag per sibling whose E2 it belongs to, and a byte per
+// sibling: the parent's E2 entries before this candidate's, were it in that
+// sibling's E2 -- all of the earlier siblings' and those of the earlier
+// candidates (216 at most).  That byte is the candidate's place among the parent's
+// E2 entries, and its place among the parent's E4 entries is
+// (sibling) |C| + (index in C) - byte.  So a warp turns 32 candidates into one
+// sibling's entries with a byte extract, a flag test, an add, an address and a
+// store -- no ballot, no population count, no cursor: the loop is bound by
+// instructions issued, not by memory.  Bytes are counted four siblings to a
+// word; a parent of up to four siblings needs one word, and is half of all
+// parents of clumped and surface-like sets.
+//
+// Entries are stored directly where the parent's lists are short.  From kStageMin
+// candidates on (and more than four siblings) four siblings' E4 entries are
+// gathered in shared memory, aligned like the output, and leave by one bulk
+// copy: DRAM and L2 see whole lines, and the loop's stores stay on chip.  Both
+// sides measured, levels 2..7 of 2^24 uniform points (216 candidates nearly
+// everywhere): 455 us gathered, 714 us stored directly; levels 2..9 of 2^24
+// points on a sphere and in clumps (60 to 100 candidates): 565 us with every
+// parent gathered, 506 us with this rule.  With one ballot, two population
+// counts and a cursor per 32 entries these took 636 and 716 us.
+//
 // kCodes: also write the E2 entries' offset codes for the next level (every
 // level but the last).
+constexpr uint32_t kStageMin = 128;   // candidates of a parent whose E4 entries are gathered first
+constexpr uint32_t kStage = 4 * 189;  // E4 entries gathered at a time: four siblings'
+struct FillWarp {
+  uint4 cand[kCand];    // rank, flags (sibling j: bit 8 j, or 8 (j - 4) + 4), bytes 0..3, 4..7
+  __align__(16) uint32_t stage[kStage + 4];
+  uint8_t pos[kCand];   // position among the children of the parent's neighbours, plus 13
+  uint8_t near[72];     // the candidates in some sibling's E2 (the 4x4x4 block)
+};
+static_assert(sizeof(FillWarp) % 16 == 0, "stage alignment");
+struct FillSmem {
+  FillWarp w[kFillWarps];
+  uint2 mask[kNbor];
+  uint32_t sel[256];    // per set of octants present: byte selectors of siblings 0..3, 4..7 << 16
+};
+
+// v to global / to shared memory (a byte address) where flag bit kBit is set /
+// clear: one test and one predicated store.
+template <uint32_t kBit>
+__device__ __forceinline__ void put_if(uint32_t* p, uint32_t v, uint32_t flags) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b32 t;\n\tand.b32 t, %2, %3;\n\tsetp.ne.u32 p, t, 0;\n\t"
+      "@p st.global.u32 [%0], %1;\n\t}" ::"l"(p), "r"(v), "r"(flags), "n"(kBit)
+      : "memory");
+}
+template <uint32_t kBit>
+__device__ __forceinline__ void put_unless(uint32_t* p, uint32_t v, uint32_t flags) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b32 t;\n\tand.b32 t, %2, %3;\n\tsetp.eq.u32 p, t, 0;\n\t"
+      "@p st.global.cs.u32 [%0], %1;\n\t}" ::"l"(p), "r"(v), "r"(flags), "n"(kBit)
+      : "memory");
+}
+template <uint32_t kBit>
+__device__ __forceinline__ void stage_unless(uint32_t p, uint32_t v, uint32_t flags) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b32 t;\n\tand.b32 t, %2, %3;\n\tsetp.eq.u32 p, t, 0;\n\t"
+      "@p st.shared.u32 [%0], %1;\n\t}" ::"r"(p), "r"(v), "r"(flags), "n"(kBit)
+      : "memory");
+}
+
+// One lane: `bytes` (a multiple of 16) from shared to global memory by a bulk
+// copy; stage_wait: the stage may be written again (and the warp's last one
+// has left shared memory).
+__device__ __forceinline__ void stage_store(uint32_t* dst, const uint32_t* src, uint32_t bytes) {
+  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n\t"
+               "cp.async.bulk.commit_group;" ::"l"(dst),
+               "r"(smem_u32(src)), "r"(bytes)
+               : "memory");
+}
+__device__ __forceinline__ void stage_wait() {
+  asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+}
+
+// Candidate e's place: the eight children of a lane's neighbour are 128 bytes
+// apart from the next lane's; swapping places inside each eight keeps the
+// lanes' stores of one octant off each other's banks.
+__device__ __forceinline__ uint32_t cand_at(uint32_t e) { return e ^ ((e >> 3) & 7u); }
+
+// f(integral_constant j) for the siblings j < nsib: of eight (more than four
+// are there), or of four.
+template <bool kWide, class F>
+__device__ __forceinline__ void each_sibling(uint32_t nsib, const F& f) {
+  f(std::integral_constant<int, 0>{});
+  if (kWide || nsib > 1) f(std::integral_constant<int, 1>{});
+  if (kWide || nsib > 2) f(std::integral_constant<int, 2>{});
+  if (kWide || nsib > 3) f(std::integral_constant<int, 3>{});
+  if constexpr (kWide) {
+    f(std::integral_constant<int, 4>{});
+    if (nsib > 5) f(std::integral_constant<int, 5>{});
+    if (nsib > 6) f(std::integral_constant<int, 6>{});
+    if (nsib > 7) f(std::integral_constant<int, 7>{});
+  }
+}
+
+// One parent: its siblings' rows and entries.  kWide: more than four siblings.
+template <bool kCodes, bool kWide>
+__device__ __forceinline__ void fill_parent(FillWarp& F, uint2 mk, uint32_t sel, uint32_t nsib,
+                                            uint32_t occ, uint32_t code, uint32_t rank,
+                                            uint32_t present, uint32_t* out2, uint32_t* out4,
+                                            uint32_t at2, uint32_t at4, uint32_t* e2, uint32_t* e4,
+                                            uint8_t* codes) {
+  const int lane = threadIdx.x & 31;
+  // child masks of the siblings, in their order; none for absent ones
+  uint32_t m0 = __byte_perm(mk.x, mk.y, sel), m1 = 0;
+  if (kWide) {
+    m1 = __byte_perm(mk.x, mk.y, sel >> 16) & (0xffffffffu >> (8u * (8u - nsib)));
+  } else {
+    m0 &= 0xffffffffu >> (8u * (4u - nsib));
+  }
+  // per lane (neighbour): candidates before it, and those in each sibling's E2
+  const uint32_t occ4 = occ * 0x01010101u;
+  const uint32_t lo0 = byte_popc(m0 & occ4), hi0 = kWide ? byte_popc(m1 & occ4) : 0u;
+  uint32_t any = (m0 | m1) & occ4;
+  any |= any >> 16;
+  any |= any >> 8;
+  const uint32_t cn = (uint32_t)__popc(occ) | ((uint32_t)__popc(any & 0xffu) << 16);
+  const uint32_t xl = warp_incl(lo0), xh = kWide ? warp_incl(hi0) : 0u;
+  const uint32_t xc = warp_incl(cn);
+  const uint32_t tl = __shfl_sync(0xffffffffu, xl, 31);
+  const uint32_t tc = __shfl_sync(0xffffffffu, xc, 31);
+  const uint32_t total = tc & 0xffffu, nnear = tc >> 16;
+  const uint32_t f0 = tl * 0x01010100u;  // E2 entries of the siblings before each
+  uint32_t f1 = 0, tw = 0;
+  if (kWide) {
+    tw = __shfl_sync(0xffffffffu, xh, 31);
+    f1 = tw * 0x01010100u + byte_sum(tl) * 0x01010101u;
+  }
+  if ((uint32_t)lane < nsib) {
+    const uint32_t f = ((kWide && lane >= 4 ? f1 : f0) >> (8 * (lane & 3))) & 0xffu;
+    out2[lane] = at2 + f;
+    out4[lane] = at4 + lane * total - f;
+  }
+  uint32_t lo = xl - lo0 + f0, hi = xh - hi0 + f1;
+  uint32_t e = (xc - cn) & 0xffffu, ne = (xc - cn) >> 16;
+#pragma unroll
+  for (int o = 0; o < 8; ++o) {
+    if ((occ >> o) & 1u) {
+      const uint32_t i0 = (m0 >> o) & 0x01010101u, i1 = kWide ? (m1 >> o) & 0x01010101u : 0u;
+      const uint32_t fl = i0 + 16u * i1;
+      F.cand[cand_at(e)] = make_uint4(rank, fl, lo, hi);
+      if (kCodes) F.pos[e] = (uint8_t)(2u * code + oct_pos(o));
+      if (fl) F.near[ne++] = (uint8_t)e;
+      ++e;
+      ++rank;
+      lo += i0;
+      if (kWide) hi += i1;
+    }
+  }
+  __syncwarp();
+  // E2: the near candidates
+  for (uint32_t i = lane; i < nnear; i += 32) {
+    const uint32_t c = F.near[i];
+    const uint4 v = F.cand[cand_at(c)];
+    const uint32_t ps = kCodes ? F.pos[c] - 13u : 0u;
+    uint32_t oct = present;  // the sibling's octant is the lowest set bit
+    each_sibling<kWide>(nsib, [&](auto jt) {
+      constexpr int j = decltype(jt)::value;
+      constexpr uint32_t bit = 1u << (j < 4 ? 8 * j : 8 * (j - 4) + 4);
+      const uint32_t x = __byte_perm(j < 4 ? v.z : v.w, 0, 0x4440 + (j & 3));
+      put_if<bit>(e2 + x, v.x, v.y);
+      if (kCodes) {  // position of the child among the parent's, less the sibling's
+        if (v.y & bit) codes[x] = (uint8_t)(ps - oct_pos(__ffs(oct) - 1));
+        oct &= oct - 1u;
+      }
+    });
+  }
+  // E4: every candidate where it is not in E2
+  if (!kWide || total < kStageMin) {
+    for (uint32_t i = lane; i < total; i += 32) {
+      const uint4 v = F.cand[cand_at(i)];
+      uint32_t at = i;
+      each_sibling<kWide>(nsib, [&](auto jt) {
+        constexpr int j = decltype(jt)::value;
+        constexpr uint32_t bit = 1u << (j < 4 ? 8 * j : 8 * (j - 4) + 4);
+        const uint32_t x = __byte_perm(j < 4 ? v.z : v.w, 0, 0x4440 + (j & 3));
+        put_unless<bit>(e4 + (at - x), v.x, v.y);
+        at += total;
+      });
+    }
+    __syncwarp();
+    return;
+  }
+  const uint32_t half = 4 * total - (f1 & 0xffu);  // E4 entries of the first four
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const uint32_t from = h ? 4 * total - half : 0u;
+    uint32_t* const dst = e4 + (h ? half : 0u);
+    const uint32_t n = h ? nsib * total - half - (f1 >> 24) - (tw >> 24) : half;
+    const uint32_t a0 = (uint32_t)(reinterpret_cast<uintptr_t>(dst) >> 2) & 3u;
+    const uint32_t base = smem_u32(F.stage) + 4u * (a0 + from);  // the stage is aligned like dst
+    for (uint32_t i = lane; i < total; i += 32) {
+      const uint4 v = F.cand[cand_at(i)];
+      const uint32_t b = h ? v.w : v.z, fl = h ? v.y >> 4 : v.y;
+      uint32_t at = base + 4u * i;
+      each_sibling<false>(h ? nsib - 4 : 4u, [&](auto jt) {
+        constexpr int j = decltype(jt)::value;
+        const uint32_t x = __byte_perm(b, 0, 0x4440 + j);
+        stage_unless<(1u << (8 * j))>(at - 4u * x, v.x, fl);
+        at += 4u * total;
+      });
+    }
+    fence_proxy_async();
+    __syncwarp();
+    // head and tail one by one, the rest by a bulk copy
+    uint32_t* const d0 = dst - a0;
+    const uint32_t a1 = a0 + n, v0 = min((a0 + 3u) & ~3u, a1), v1 = max(a1 & ~3u, v0);
+    if (lane == 0 && v1 > v0) stage_store(d0 + v0, F.stage + v0, 4u * (v1 - v0));
+    if ((uint32_t)lane < v0 - a0) d0[a0 + lane] = F.stage[a0 + lane];
+    if ((uint32_t)lane < a1 - v1) d0[v1 + lane] = F.stage[v1 + lane];
+    if (lane == 0) stage_wait();
+    __syncwarp();
+  }
+}
+
 template <bool kCodes>
-__global__ void __launch_bounds__(kListThreads, 4) list_fill_kernel(const Seg* __restrict__ segs,
-                                                                const Job* __restrict__ jobs,
-                                                                uint32_t njobs, int l,
-                                                                const ListLevel* lvls,
-                                                                DevStatus* st) {
-  __shared__ uint32_t s_rank[kListWarps][kCand];
-  // per candidate: its sibling byte, and above it (lane of its neighbour) * 8 + octant
-  __shared__ uint16_t s_sib[kListWarps][kCand];
-  __shared__ uint32_t s_nrank[kListWarps][kNear];
-  __shared__ uint16_t s_nsib[kListWarps][kNear];
-  __shared__ WarpJob s_job[kListWarps];
-  __shared__ __align__(16) uint32_t s_stage[kListWarps][kStage];  // E4 lists of four siblings
+__global__ void __launch_bounds__(kListThreads, 4) list_fill_kernel(
+    const Seg* __restrict__ segs, const Job* __restrict__ jobs, uint32_t njobs, int l,
+    const __grid_constant__ ListLevel LV, const __grid_constant__ ListLevel up, DevStatus* st) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  FillSmem& sm = *reinterpret_cast<FillSmem*>(smem_raw);
+  __shared__ WarpJob s_job[kFillWarps];
   if (failed(st)) return;  // set before this launch: the same for every thread
-  const ListLevel& LV = lvls[l];
-  if ((LV.total[0] >> 32) != 0 || (LV.total[1] >> 32) != 0) return;  // capacity error set
-  // The level's arrays in registers: the list stores must not force reloads
-  // of the descriptor.
-  const uint32_t* const jprefix = LV.jprefix;
-  const uint32_t* const work2 = LV.work2;
-  const uint32_t* const work4 = LV.work4;
-  uint32_t* const idx2 = LV.idx2;
-  uint32_t* const idx4 = LV.idx4;
-  uint64_t* const lbase = LV.base;
-  uint64_t* const lnnz = LV.nnz;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint32_t lt = lanemask_lt();
-  uint32_t* crank = s_rank[warp];
-  uint16_t* csib = s_sib[warp];
-  uint32_t* nrank = s_nrank[warp];
-  uint16_t* nsibm = s_nsib[warp];
-  uint32_t* stage = s_stage[warp];
-  uint8_t* const code2 = LV.code2;
-  const uint32_t npar = jprefix[njobs];
-  const BlockRange br = block_range(npar);
-  // The warp's current job lives in shared memory, not in registers: the
-  // list loops below need the registers for the eight siblings' cursors.
-  WarpJob& J = s_job[warp];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t chunks = njobs == 1 ? job_chunks(jobs[0], segs, l) : LV.jchunks[njobs];
+  // A warp takes whole chunks, or in small levels a part of one.
+  const uint32_t warps = gridDim.x * kFillWarps;
+  const uint32_t split = 4u * chunks <= warps ? 4u : (2u * chunks <= warps ? 2u : 1u);
+  if (blockIdx.x * kFillWarps >= chunks * split) return;
+  if (tid < kNbor) sm.mask[tid] = code_masks(tid);
+  for (int t = tid; t < 256; t += kListThreads) {
+    uint32_t sel = 0, n = 0;
+    for (uint32_t rho = 0; rho < 8; ++rho)
+      if ((t >> rho) & 1) sel |= rho << (4 * n++);
+    sm.sel[t] = sel;
+  }
+  __syncthreads();
+  const uint32_t range = count_range(chunks);
+  FillWarp& F = sm.w[warp];
+  WarpJob& W = s_job[warp];
   uint32_t jend = 0;
-  for (uint32_t g = br.g0 + warp; g < br.g1; g += kListWarps) {
-    if (g >= jend) {  // g only grows: look its job up when it leaves the current one
+  for (uint32_t u = blockIdx.x * kFillWarps + warp; u < chunks * split; u += warps) {
+    const uint32_t c = u / split;  // (a power of two)
+    if (c >= jend) {  // c only grows
       if (lane == 0) {
-        const uint32_t j = find_job(jprefix, njobs, g);
-        J.a = make_ctx(segs, jobs[j], l, lvls, j);
-        J.j = j;
-        J.jstart = jprefix[j];
-        J.jend = jprefix[j + 1];
-        J.out2 = jobs[j].out2[l];
-        J.out4 = jobs[j].out4[l];
-        J.G2 = work2[J.a.region];
-        J.G4 = work4[J.a.region];
-        J.big = work4[J.a.region + J.a.nrecv] - J.G4 >= kStageJob;
+        load_job(W, segs, jobs, njobs, l, LV, up, c);
+        W.base2 = LV.jbase[2 * W.j];
+        W.base4 = LV.jbase[2 * W.j + 1];
       }
       __syncwarp();
-      jend = J.jend;
+      jend = W.chunk1;
     }
-    const uint32_t p = g - J.jstart;
-    const uint32_t region = J.a.region, G2 = J.G2, G4 = J.G4;
-    const bool big = J.big != 0;
-    uint32_t* const out2 = J.out2;
-    uint32_t* const out4 = J.out4;
-    // The receiver children of p (at most 8): lane j fetches child j's octant
-    // and list starts up front, so their loads overlap the neighbour loads.
-    const uint32_t c0 = J.a.rchild_up[p];
-    const uint32_t c1 = min(J.a.rchild_up[p + 1], c0 + 8u);  // (at most 8 in a whole tree)
-    uint32_t my_rho = 0, my_o2 = 0, my_o4 = 0;
-    if (c0 + lane < c1) {
-      my_rho = (uint32_t)(J.a.rkey[c0 + lane] & 7u);
-      my_o2 = work2[region + c0 + lane];
-      my_o4 = work4[region + c0 + lane];
-      out2[c0 + lane] = my_o2 - G2;
-      out4[c0 + lane] = my_o4 - G4;
+    const uint32_t p0 = (c - W.chunk0) * kChunk, np = W.np;
+    // 1. The chunk's parents, every load of one step of the chain (row start ->
+    // entry -> child and occupancy) in flight together.
+    // lanes 0..4: E2 rows of the level above, 8..12: children, 16..19 / 24..27:
+    // first E2 / E4 entries
+    const int sub = lane >> 3, l8 = lane & 7;
+    uint32_t head = 0;
+    if (sub < 2 ? l8 <= kChunk : l8 < kChunk) {
+      const uint32_t* src;
+      if (sub == 0)
+        src = l == 2 ? nullptr : W.off_up + min(p0 + l8, np);
+      else if (sub == 1)
+        src = W.rchild + min(p0 + l8, np);
+      else
+        src = (sub == 2 ? LV.off2 : LV.off4) + (uint64_t)c * kChunk + l8;
+      if (src) head = *src;
     }
-    if (g + 1 == jend) {  // the job's last parent closes its rows
-      const uint32_t nrecv = J.a.nrecv, j = J.j;
-      const uint32_t e2 = work2[region + nrecv], e4 = work4[region + nrecv];
-      if (lane == 0) {
-        out2[nrecv] = e2 - G2;
-        out4[nrecv] = e4 - G4;
-        lbase[2 * j] = G2;
-        lbase[2 * j + 1] = G4;
-        lnnz[2 * j] = e2 - G2;
-        lnnz[2 * j + 1] = e4 - G4;
-      }
-    }
-    const Neighbour q = load_neighbour(J.a, l, p, lane);
-    const uint32_t nsib = c1 - c0;
-    // this lane's neighbour's part of the position sum P (see the E2 loop)
-    const int pbase = (2 * q.dx + 1) + 3 * (2 * q.dy + 1) + 9 * (2 * q.dz + 1);
-
-    // Candidates C (children of p's neighbours, ascending rank) and the near
-    // candidates (those in some sibling's E2), each with its sibling byte.
-    const uint32_t nc = __popc(q.occ);
-    uint32_t e = warp_excl(nc, lane);
-    const uint32_t total = __shfl_sync(0xffffffffu, e + nc, 31);
+    const uint64_t g2 = LV.bbase[2 * (c / range)] - W.base2;  // (job-relative)
+    const uint64_t g4 = LV.bbase[2 * (c / range) + 1] - W.base4;
+    uint32_t cc[kChunk], ch[kChunk];  // occupancy | code << 8, first child
     {
-      // The sibling byte of child o of this neighbour factors by axis: bit
-      // rho is set iff axis_mask(-delta, o's bit, ...) holds on every axis.
-      // Branch-free over the eight octants (predicated stores).
-      const uint32_t mx0 = axis_mask(-q.dx, 0u, 0x55u, 0xaau), mx1 = axis_mask(-q.dx, 1u, 0x55u, 0xaau);
-      const uint32_t my0 = axis_mask(-q.dy, 0u, 0x33u, 0xccu), my1 = axis_mask(-q.dy, 1u, 0x33u, 0xccu);
-      const uint32_t mz0 = axis_mask(-q.dz, 0u, 0x0fu, 0xf0u), mz1 = axis_mask(-q.dz, 1u, 0x0fu, 0xf0u);
-      uint32_t rank = q.child;
-      const uint32_t lane8 = (uint32_t)lane << 11;  // (lane * 8) << 8
+      uint32_t q[kChunk];
+      bool in[kChunk];
 #pragma unroll
-      for (int o = 0; o < 8; ++o) {
-        if ((q.occ >> o) & 1u) {
-          crank[e] = rank++;
-          csib[e] = (uint16_t)((((o & 1) ? mx1 : mx0) & ((o & 2) ? my1 : my0) & ((o & 4) ? mz1 : mz0)) |
-                               lane8 | ((uint32_t)o << 8));
-          ++e;
-        }
-      }
-    }
-    __syncwarp();
-    uint32_t nnear = 0;
-    for (uint32_t c = 0; c < total; c += 32) {
-      const uint32_t i = c + lane;
-      const uint32_t sb16 = i < total ? csib[i] : 0u;
-      const bool near = (sb16 & 0xffu) != 0u;
-      const uint32_t bn = __ballot_sync(0xffffffffu, near);
-      if (near) {
-        const uint32_t k = nnear + __popc(bn & lt);
-        nrank[k] = crank[i];
-        nsibm[k] = (uint16_t)sb16;
-      }
-      nnear += __popc(bn);
-    }
-    __syncwarp();
-
-    uint32_t sbit[8], w2[8], w4[8];
-#pragma unroll
-    for (int jj = 0; jj < 8; ++jj) {
-      sbit[jj] = 1u << __shfl_sync(0xffffffffu, my_rho, jj);
-      w2[jj] = __shfl_sync(0xffffffffu, my_o2, jj);
-      w4[jj] = __shfl_sync(0xffffffffu, my_o4, jj);
-    }
-    // E2 of sibling jj: the near candidates whose byte has bit rho_jj; E4:
-    // the candidates without it.  A parent with all eight children runs the
-    // eight siblings as straight-line code; otherwise absent siblings (the
-    // same for the whole warp) are skipped.
-    auto emit = [&](auto all_tag) {
-      constexpr bool kAll = decltype(all_tag)::value;
-      for (uint32_t c = 0; c < nnear; c += 32) {
-        const uint32_t i = c + lane;
-        const uint32_t v = i < nnear ? nrank[i] : 0u;
-        const uint32_t sb16 = i < nnear ? nsibm[i] : 0u;
-        const uint32_t sb = sb16 & 0xffu;
-        // Position of the candidate, child o of the neighbour at delta, among
-        // the parent's children: p = 2 delta + o per axis; P = sum over axes of
-        // 3^axis (p + 1).  Minus the sibling's (rx + 3 ry + 9 rz) it is the
-        // entry's offset code (dx+1) + 3(dy+1) + 9(dz+1) from that sibling.
-        uint32_t P = 0;
-        if (kCodes) {
-          const uint32_t cq = sb16 >> 8, o = cq & 7u;
-          P = (uint32_t)__shfl_sync(0xffffffffu, pbase, (int)(cq >> 3)) + (o & 1u) +
-              3u * ((o >> 1) & 1u) + 9u * (o >> 2);
-        }
-#pragma unroll
-        for (int jj = 0; jj < 8; ++jj) {
-          if (kAll || (uint32_t)jj < nsib) {
-            const uint32_t hit = sb & sbit[jj];
-            const uint32_t b2 = __ballot_sync(0xffffffffu, hit != 0u);
-            const uint32_t at = w2[jj] + __popc(b2 & lt);
-            st_cs_if(idx2 + at, v, hit);
-            if (kCodes) {
-              const uint32_t rho = __ffs(sbit[jj]) - 1u;
-              const uint32_t R = (rho & 1u) + 3u * ((rho >> 1) & 1u) + 9u * (rho >> 2);
-              if (hit) code2[at] = (uint8_t)(P - R);
-            }
-            w2[jj] += __popc(b2);
+      for (int k = 0; k < kChunk; ++k) {
+        const uint32_t first = __shfl_sync(0xffffffffu, head, k);
+        const uint32_t end = __shfl_sync(0xffffffffu, head, k + 1);
+        const uint32_t m = l == 2 ? (p0 + k < np ? W.nsrc1 : 0u) : min(end - first, (uint32_t)kNbor);
+        in[k] = (uint32_t)lane < m;
+        q[k] = lane;
+        cc[k] = 13u << 8;
+        if (in[k]) {
+          if (l == 2) {
+            cc[k] = level1_code((uint32_t)segs[jobs[W.j].src].lv.key[1][lane],
+                                (uint32_t)segs[jobs[W.j].recv].lv.key[1][p0 + k])
+                    << 8;
+          } else {
+            q[k] = W.idx_up[first + lane];
+            cc[k] = (uint32_t)W.code_up[first + lane] << 8;
           }
         }
       }
-      // E4.  Where a job's E4 lists of the level outgrow L2, a parent with all eight
-      // children and many candidates gathers its E4 lists four siblings at a
-      // time in the warp's stage (they are adjacent in idx4; the stage is
-      // aligned like idx4) and writes them as whole 16-byte vectors, so that
-      // DRAM sees whole sectors; elsewhere the entries are stored directly
-      // (partial writes merge in L2 there).
-      if (kAll && big && total >= kStageMin) {
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const uint32_t a0 = w4[4 * h], sb0 = a0 & ~3u;
-          for (uint32_t c = 0; c < total; c += 32) {
-            const uint32_t i = c + lane;
-            const uint32_t v = i < total ? crank[i] : 0u;
-            const uint32_t sb = i < total ? (csib[i] & 0xffu) : 0xffu;  // past the end: never stored
-#pragma unroll
-            for (int jj = 4 * h; jj < 4 * h + 4; ++jj) {
-              const uint32_t hit = sb & sbit[jj];
-              const uint32_t b4 = __ballot_sync(0xffffffffu, hit == 0u);
-              const uint32_t at = w4[jj] + __popc(b4 & lt) - sb0;
-              if (hit == 0u && at < kStage) stage[at] = v;
-              w4[jj] += __popc(b4);
-            }
-          }
-          __syncwarp();
-          // the half's entries [a0, a1): head and tail one by one, the rest
-          // as 16-byte vectors
-          const uint32_t a1 = w4[4 * h + 3];
-          const uint32_t v0 = min((a0 + 3u) & ~3u, a1), v1 = max(a1 & ~3u, v0);
-          if ((uint32_t)lane < v0 - a0) __stcs(idx4 + a0 + lane, stage[a0 + lane - sb0]);
-          if ((uint32_t)lane < a1 - v1) __stcs(idx4 + v1 + lane, stage[v1 + lane - sb0]);
-          for (uint32_t e = v0 + 4u * lane; e < v1; e += 128u)
-            __stcs(reinterpret_cast<uint4*>(idx4 + e),
-                   *reinterpret_cast<const uint4*>(stage + (e - sb0)));
-          __syncwarp();
-        }
-      } else {
-        for (uint32_t c = 0; c < total; c += 32) {
-          const uint32_t i = c + lane;
-          const uint32_t v = i < total ? crank[i] : 0u;
-          const uint32_t sb = i < total ? (csib[i] & 0xffu) : 0xffu;  // past the end: never stored
-#pragma unroll
-          for (int jj = 0; jj < 8; ++jj) {
-            if (kAll || (uint32_t)jj < nsib) {
-              const uint32_t hit = sb & sbit[jj];
-              const uint32_t b4 = __ballot_sync(0xffffffffu, hit == 0u);
-              st_cs_if_zero(idx4 + w4[jj] + __popc(b4 & lt), v, hit);
-              w4[jj] += __popc(b4);
-            }
-          }
-        }
+      for (int k = 0; k < kChunk; ++k) {
+        cc[k] |= in[k] ? W.socc[q[k]] : 0u;
+        ch[k] = in[k] ? W.schild[q[k]] : 0u;
       }
-    };
-    if (nsib == 8)
-      emit(std::true_type{});
-    else
-      emit(std::false_type{});
-    __syncwarp();
+    }
+    uint32_t octs;  // lanes 8 k ..: octants of parent k's receiver children
+    {
+      const uint32_t r0 = __shfl_sync(0xffffffffu, head, 8 + sub);
+      const uint32_t nch = min(__shfl_sync(0xffffffffu, head, 9 + sub) - r0, 8u);
+      octs = (uint32_t)l8 < nch ? 1u << (uint32_t)(W.rkey[r0 + l8] & 7u) : 0u;
+#pragma unroll
+      for (int o = 1; o < 8; o <<= 1) octs |= __shfl_xor_sync(0xffffffffu, octs, o);
+    }
+    // 2. The parents, one after another.
+    const uint32_t k0 = (u % split) * (kChunk / split), k1 = min(k0 + kChunk / split, np - p0);
+    for (uint32_t k = 0; k < k1; ++k) {
+      const uint32_t co = cc[0], rank = ch[0];
+#pragma unroll
+      for (int i = 0; i + 1 < kChunk; ++i) {
+        cc[i] = cc[i + 1];
+        ch[i] = ch[i + 1];
+      }
+      if (k < k0) continue;
+      const uint32_t present = __shfl_sync(0xffffffffu, octs, 8 * k);
+      const uint32_t c0 = __shfl_sync(0xffffffffu, head, 8 + k);
+      const uint64_t at2 = g2 + __shfl_sync(0xffffffffu, head, 16 + k);
+      const uint64_t at4 = g4 + __shfl_sync(0xffffffffu, head, 24 + k);
+      const uint32_t nsib = __popc(present);
+      const uint64_t slot = W.slot;
+      uint32_t* const e2 = LV.idx2 + 27ull * slot + at2;
+      uint32_t* const e4 = LV.idx4 + 189ull * slot + at4;
+      uint8_t* const codes = kCodes ? LV.code2 + 27ull * slot + at2 : nullptr;
+      const uint2 mk = sm.mask[co >> 8];
+      const uint32_t sel = sm.sel[present];
+      if (nsib > 4)
+        fill_parent<kCodes, true>(F, mk, sel, nsib, co & 0xffu, co >> 8, rank, present,
+                                  W.out2 + c0, W.out4 + c0, (uint32_t)at2, (uint32_t)at4, e2, e4,
+                                  codes);
+      else if (nsib > 0)
+        fill_parent<kCodes, false>(F, mk, sel, nsib, co & 0xffu, co >> 8, rank, present,
+                                   W.out2 + c0, W.out4 + c0, (uint32_t)at2, (uint32_t)at4, e2, e4,
+                                   codes);
+    }
   }
 }
 
 void launch_list_count(const Seg* segs, const Job* jobs, uint32_t njobs, int l,
-                       const ListLevel* lvls, DevStatus* st, cudaStream_t s) {
-  list_count_kernel<<<152u * 8u, kListThreads, 0, s>>>(segs, jobs, njobs, l, lvls, st);
+                       const ListLevel& lv, const ListLevel& up, uint32_t max_chunks, DevStatus* st,
+                       cudaStream_t s) {
+  const uint32_t grid = std::min((max_chunks + kCountWarps - 1) / kCountWarps, kCountGrid);
+  list_count_kernel<<<std::max(grid, 1u), kListThreads, 0, s>>>(segs, jobs, njobs, l, lv, up, st);
 }
 
 void launch_list_fill(const Seg* segs, const Job* jobs, uint32_t njobs, int l,
-                      const ListLevel* lvls, bool codes, DevStatus* st, cudaStream_t s) {
-  if (codes)
-    list_fill_kernel<true><<<152u * 8u, kListThreads, 0, s>>>(segs, jobs, njobs, l, lvls, st);
+                      const ListLevel& lv, const ListLevel& up, uint32_t max_chunks, DevStatus* st,
+                      cudaStream_t s) {
+  static const bool attr = [] {
+    cudaFuncSetAttribute(list_fill_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)sizeof(FillSmem));
+    cudaFuncSetAttribute(list_fill_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)sizeof(FillSmem));
+    return true;
+  }();
+  (void)attr;
+  const uint64_t units = 4ull * max_chunks;  // a warp takes one parent at least
+  const uint32_t grid = (uint32_t)std::max<uint64_t>(
+      std::min<uint64_t>((units + kFillWarps - 1) / kFillWarps, kFillGrid), 1u);
+  if (lv.code2)
+    list_fill_kernel<true><<<grid, kListThreads, sizeof(FillSmem), s>>>(segs, jobs, njobs, l, lv, up, st);
   else
-    list_fill_kernel<false><<<152u * 8u, kListThreads, 0, s>>>(segs, jobs, njobs, l, lvls, st);
+    list_fill_kernel<false><<<grid, kListThreads, sizeof(FillSmem), s>>>(segs, jobs, njobs, l, lv, up, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -623,16 +794,8 @@ __host__ __device__ inline uint32_t scan_tiles_of(uint32_t cap) {
 
 uint32_t scan_tiles(uint32_t cap) { return scan_tiles_of(cap); }
 
-// Up to two arrays of the same length in one launch (the E2 and E4 counts of
-// a level): tickets [0, need) scan the first, [need, 2 need) the second, each
-// with its own look-back words and total.
-struct ScanArray {
-  uint32_t* data;
-  uint64_t* status;
-  uint64_t* total64;
-};
-
-__global__ void __launch_bounds__(kScanThreads) scan_u32_kernel(ScanArray a0, ScanArray a1,
+__global__ void __launch_bounds__(kScanThreads) scan_u32_kernel(uint32_t* data, uint64_t* status,
+                                                               uint64_t* total64,
                                                                const uint32_t* count_dev,
                                                                uint32_t cap, uint32_t* counter,
                                                                DevStatus* st, uint64_t wait_ns) {
@@ -644,13 +807,8 @@ __global__ void __launch_bounds__(kScanThreads) scan_u32_kernel(ScanArray a0, Sc
   const uint32_t need = scan_tiles_of(count);
   if (threadIdx.x == 0) s_tile = atomicAdd(counter, 1u);
   __syncthreads();
-  const uint32_t ticket = s_tile;
-  const bool second = ticket >= need;
-  if (second && (a1.data == nullptr || ticket >= 2 * need)) return;
-  const uint32_t tile = second ? ticket - need : ticket;
-  uint32_t* const data = second ? a1.data : a0.data;
-  uint64_t* const status = second ? a1.status : a0.status;
-  uint64_t* const total64 = second ? a1.total64 : a0.total64;
+  const uint32_t tile = s_tile;
+  if (tile >= need) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint64_t i0 = (uint64_t)tile * kScanTile + (uint64_t)threadIdx.x * kScanItems;
   uint32_t v[kScanItems];
@@ -739,17 +897,8 @@ __global__ void __launch_bounds__(kScanThreads) scan_u32_kernel(ScanArray a0, Sc
 void launch_scan_u32(uint32_t* data, const uint32_t* count_dev, uint32_t cap, uint64_t* status,
                      uint32_t* counter, uint64_t* total64, DevStatus* st, uint64_t wait_ns,
                      cudaStream_t s) {
-  scan_u32_kernel<<<scan_tiles(cap), kScanThreads, 0, s>>>(ScanArray{data, status, total64},
-                                                           ScanArray{nullptr, nullptr, nullptr},
-                                                           count_dev, cap, counter, st, wait_ns);
-}
-
-void launch_scan_u32_pair(uint32_t* data0, uint64_t* status0, uint64_t* total0, uint32_t* data1,
-                          uint64_t* status1, uint64_t* total1, uint32_t cap, uint32_t* counter,
-                          DevStatus* st, uint64_t wait_ns, cudaStream_t s) {
-  scan_u32_kernel<<<2 * scan_tiles(cap), kScanThreads, 0, s>>>(
-      ScanArray{data0, status0, total0}, ScanArray{data1, status1, total1}, nullptr, cap, counter,
-      st, wait_ns);
+  scan_u32_kernel<<<scan_tiles(cap), kScanThreads, 0, s>>>(data, status, total64, count_dev, cap,
+                                                           counter, st, wait_ns);
 }
 
 }  // namespace fmm
