@@ -2009,36 +2009,31 @@ int fmm_box_types(fmm_ctx* c, const fmm_tree* t, int lpar, const uint32_t* owner
   cudaStream_t s = c->stream;
   int err = FMM_OK;
   const int L = t->L, lcrit = std::max(lpar - 1, 2);
-  std::vector<uint8_t*> on(kLevels, nullptr);
+  // Levels lpar..L: on-J flags, and which boxes' E2 crosses J's border.
+  std::vector<uint8_t*> on(kLevels, nullptr), border(kLevels, nullptr);
   for (int l = lpar; l <= L; ++l) {
     on[l] = arena_get<uint8_t>(c, t->nbox_src[l], &err);
-    if (err) return err;
-    Launch Lk(c, "box_types");
-    launch_on_node(l == lpar ? owner : nullptr, t->parent_src[l], on[l - 1], t->nbox_src[l], node,
-                   on[l], s);
+    border[l] = arena_get<uint8_t>(c, t->nbox_src[l], &err);
   }
-  uint8_t* sides = nullptr;
-  if (lcrit < lpar) {
-    sides = arena_get<uint8_t>(c, t->nbox_src[lcrit], &err);
-    if (err) return err;
+  // child sides of the lcrit boxes: bit 0 a descendant at lpar on J, bit 1 one
+  // off J (lcrit = lpar = 2: the box itself)
+  uint8_t* sides = arena_get<uint8_t>(c, t->nbox_src[lcrit], &err);
+  if (err) return err;
+  {
     Launch Lk(c, "box_types");
-    launch_child_sides(t->child_src[lcrit], on[lpar], t->nbox_src[lcrit], sides, s);
+    launch_on_node(owner, t->nbox_src[lpar], node, on[lpar], s);
+  }
+  {
+    Launch Lk(c, "box_types");
+    launch_child_sides(lcrit < lpar ? t->child_src[lcrit] : nullptr, on[lpar], t->nbox_src[lcrit],
+                       sides, s);
   }
   for (int l = 2; l <= L; ++l) {
     Launch Lk(c, "box_types");
-    if (l < lcrit) {
-      launch_box_type(nullptr, nullptr, nullptr, nullptr, t->nbox_src[l], 0, types[l], s);
-    } else if (l == lcrit && lcrit < lpar) {
-      launch_box_type(t->e4_off[l], t->e4_idx[l], sides, nullptr, t->nbox_src[l], 1, types[l], s);
-    } else if (l == lcrit) {  // lcrit = lpar = 2: a box's own ownership decides
-      // its descendants at lpar are itself: bit 0 on J, bit 1 off J
-      uint8_t* sd = arena_get<uint8_t>(c, t->nbox_src[l], &err);
-      if (err) return err;
-      launch_child_sides(nullptr, on[l], t->nbox_src[l], sd, s);
-      launch_box_type(t->e4_off[l], t->e4_idx[l], sd, nullptr, t->nbox_src[l], 1, types[l], s);
-    } else {
-      launch_box_type(t->e4_off[l], t->e4_idx[l], nullptr, on[l], t->nbox_src[l], 2, types[l], s);
-    }
+    const int mode = l < lcrit ? 0 : (l == lcrit ? 1 : 2);
+    launch_box_type(*t, l, mode, mode == 1 ? sides : on[l], on[l],
+                    l > lpar ? border[l - 1] : nullptr, border[l],
+                    l >= lpar && l < L ? on[l + 1] : nullptr, types[l], s);
   }
   FMM_CUDA(cudaGetLastError());
   return FMM_OK;
