@@ -346,6 +346,59 @@ constexpr int kBkHistLevels = 3;
 constexpr int kBkHistCells = 8 + 64 + 512;
 __device__ __forceinline__ int hoff(int m) { return ((1 << (3 * m)) - 8) / 7; }
 
+// A sub-cell, whose order and boxes one block makes: found by one thread, read by
+// the block from shared memory (in every thread's registers it spilled: 363 us
+// for the 8192 sub-cells of 2 x 2^24 uniform points, 395 us so).
+struct BoxJob {
+  const uint64_t* items;  // its items
+  const float* xyz;
+  uint64_t* status;       // [kLevels][nsub] look-back words of the set
+  uint64_t keep;          // key bits an item keeps, in place
+  uint32_t n, off;        // points, bookmark
+  uint32_t u, nsub;       // place in the set's chain, chain length
+  uint32_t key, d0;       // cell key; first level at which its first point opens a box
+  int lev, Lb, ib, D;     // cell level, box depth, index bits, group bits
+  bool last, trunc;       // the set's last one; items hold fewer key bits than lie below the cell
+  uint32_t seg, more;     // the set's Seg; a sub-cell was found
+};
+
+// The sub-cell of ticket t (one thread).
+__device__ void find_box_job(const BkSet* bsets, const Slot* slots, uint32_t nslots, uint32_t t,
+                             BoxJob& S) {
+  const Slot sl = slots[find_slot(slots, nslots, t)];
+  const BkSet& K = bsets[sl.seg];
+  S.u = t - sl.unit0;  // sub-cell slot of the set: bucket b, octant j
+  const uint32_t b = S.u >> 3, j = S.u & 7u;
+  const uint32_t nbk = K.info[0];
+  if (b >= nbk) return;  // past the set's last non-empty cell
+  S.seg = K.seg;
+  S.xyz = K.xyz;
+  S.lev = K.bl + 1;
+  S.Lb = K.Lb;
+  S.ib = K.ib;
+  S.D = K.D;
+  S.keep = K.keep << 3;
+  S.trunc = K.trunc != 0;
+  S.nsub = 8 * K.nslot;
+  S.status = K.status;
+  S.n = K.scnt[S.u];
+  S.off = K.soff[S.u];
+  const uint32_t cell = K.bcell[b];
+  S.key = cell * 8 + j;
+  S.items = K.items + (uint64_t)S.key * kBkCap;
+  S.last = b == nbk - 1 && j == 7;
+  // The first point of the sub-cell opens a box at every level from the
+  // first one at which it differs from the point before it in the set.
+  S.d0 = 0;
+  if (S.off > K.boff[b]) {  // a non-empty sub-cell precedes this one in the bucket
+    S.d0 = (uint32_t)S.lev;
+  } else if (b > 0) {
+    const uint32_t x = cell ^ K.bcell[b - 1];  // non-zero: distinct cells
+    S.d0 = (uint32_t)K.bl - (uint32_t)(31 - __clz((int)x)) / 3u;
+  }
+  S.more = 1;
+}
+
 __global__ void __launch_bounds__(kBkThreads, 3) bucket_boxes_kernel(
     const BkSet* __restrict__ bsets, const Seg* __restrict__ segs, const Slot* __restrict__ slots,
     uint32_t nslots, uint32_t* ticket, DevStatus* st, uint64_t wait_ns) {
@@ -362,39 +415,23 @@ __global__ void __launch_bounds__(kBkThreads, 3) bucket_boxes_kernel(
   __shared__ uint64_t* s_lkey[kLevels];                  // the output level arrays
   __shared__ uint32_t *s_loff[kLevels], *s_lpar[kLevels], *s_lchd[kLevels];
   __shared__ uint32_t s_lcap[kLevels];
+  __shared__ BoxJob S;
 
   const int tid = threadIdx.x, lane = tid & 31;
   if (tid == 0) {
-    s_t = atomicAdd(ticket, 1u);
     s_abort = failed(st) ? 1u : 0u;
+    S.more = 0;
+    if (!s_abort) find_box_job(bsets, slots, nslots, atomicAdd(ticket, 1u), S);
   }
   __syncthreads();
-  if (s_abort) return;  // an earlier kernel failed: leave the outputs alone
-  const uint32_t t = s_t;
-  const Slot sl = slots[find_slot(slots, nslots, t)];
-  const BkSet& S = bsets[sl.seg];
-  const uint32_t u = t - sl.unit0;  // sub-cell slot of the set: bucket b, octant j
-  const uint32_t b = u >> 3, j = u & 7u;
-  const uint32_t nbk = S.info[0];
-  if (b >= nbk) return;  // past the set's last non-empty cell
+  // an earlier kernel failed (the outputs are left alone), or past the last one
+  if (s_abort || !S.more) return;
   const Seg& G = segs[S.seg];
-  const int bl = S.bl, bl1 = bl + 1, Lb = S.Lb, ib = S.ib, D = S.D;
-  const uint64_t imask = (1ull << ib) - 1ull, keep1 = S.keep << 3;
-  const uint32_t nsub = 8 * S.nslot;
+  const int bl1 = S.lev, Lb = S.Lb, ib = S.ib, D = S.D;
+  const uint64_t imask = (1ull << ib) - 1ull, keep1 = S.keep;
+  const uint32_t nsub = S.nsub, u = S.u, d0 = S.d0;
   uint64_t* const status = S.status;  // [kLevels][nsub]: one chain of sub-cells per level
-  const uint32_t n_j = S.scnt[u], offj = S.soff[u];
-  const uint32_t cell = S.bcell[b], cell1 = cell * 8 + j;
-  // a non-empty sub-cell precedes this one in the bucket
-  const bool sib = __syncthreads_or(tid < (int)j && S.scnt[8 * b + tid] > 0);
-  // The first point of the sub-cell opens a box at every level from the
-  // first one at which it differs from the point before it in the set.
-  uint32_t d0 = 0;
-  if (sib) {
-    d0 = (uint32_t)bl1;
-  } else if (b > 0) {
-    const uint32_t x = cell ^ S.bcell[b - 1];  // non-zero: distinct cells
-    d0 = (uint32_t)bl - (uint32_t)(31 - __clz((int)x)) / 3u;
-  }
+  const uint32_t n_j = S.n, offj = S.off, cell1 = S.key;
   if (n_j > (uint32_t)kBkCap) {
     // More points than a block sorts: the host builds this set again by the
     // radix path.  The build stops here (later kernels see the status and
@@ -422,7 +459,7 @@ __global__ void __launch_bounds__(kBkThreads, 3) bucket_boxes_kernel(
 
   // 1. The sub-cell's items (all loads in flight together; kept in L2 for
   // the counting sort's scatter, which reads them again).
-  const uint64_t* src = S.items + (uint64_t)cell1 * kBkCap;
+  const uint64_t* src = S.items;
   const uint32_t ng = 1u << D;
   const int gsh = 64 - D;
   uint32_t rk[kBkItems];
@@ -620,11 +657,11 @@ __global__ void __launch_bounds__(kBkThreads, 3) bucket_boxes_kernel(
   // 7. Outputs: the set's totals (last sub-cell slot of the last bucket);
   // the boxes starting at point 0 at levels <= bl1; the boxes of levels
   // bl1 + 1 .. lh, one thread per cell; the deeper boxes.
-  if (b == nbk - 1 && j == 7 && tid <= Lb) {
+  if (S.last && tid <= Lb) {
     const uint32_t tot = s_R[tid] + s_C[tid];
     G.nbox[tid] = tot;
     if (tot <= s_lcap[tid]) {
-      s_loff[tid][tot] = S.n;
+      s_loff[tid][tot] = G.n;
       if (tid < Lb) s_lchd[tid][tot] = s_R[tid + 1] + s_C[tid + 1];
     }
   }
