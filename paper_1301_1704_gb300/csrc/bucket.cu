@@ -118,9 +118,9 @@ __global__ void __launch_bounds__(kBkPlanThreads) bucket_plan_kernel(const BkSet
       const uint4 lo = *reinterpret_cast<const uint4*>(S.sct + 8 * (c0 + k));
       const uint4 hi = *reinterpret_cast<const uint4*>(S.sct + 8 * (c0 + k) + 4);
       v[k] = lo.x + lo.y + lo.z + lo.w + hi.x + hi.y + hi.z + hi.w;
+      mx = max(mx, max(max(max(lo.x, lo.y), max(lo.z, lo.w)), max(max(hi.x, hi.y), max(hi.z, hi.w))));
     }
     sum += (uint64_t)v[k] | ((uint64_t)(v[k] != 0) << 32);
-    mx = v[k] > mx ? v[k] : mx;
   }
   uint64_t x = sum;
 #pragma unroll
@@ -147,8 +147,15 @@ __global__ void __launch_bounds__(kBkPlanThreads) bucket_plan_kernel(const BkSet
     }
     const uint32_t nbk = (uint32_t)(run >> 32);
     S.info[0] = nbk;
-    S.info[1] = m;
     S.boff[nbk] = S.n;
+    if (S.info[2]) {
+      // A sub-cell is too full for one block: the host builds the set again by
+      // the radix passes, to a depth that follows from the fullest sub-cell
+      // (scaled up: the scatter stopped once it had found one).
+      const uint64_t all = max(run & 0xffffffffull, 1ull);
+      S.info[1] = (uint32_t)min((uint64_t)S.n, (uint64_t)m * S.n / all);
+      set_error(st, kStatusBucketFull);
+    }
   }
   __syncthreads();
   uint64_t e = s_w[warp] + x - sum;
@@ -211,7 +218,8 @@ __global__ void __launch_bounds__(kScThreads, 1) bucket_scatter_kernel(
   const int sh = 63 - 3 * bl1, lsh = 1 + 3 * bl1;
   const uint64_t keep1 = S.keep << 3;
   for (uint32_t c = threadIdx.x; c < subs; c += blockDim.x) s_at[c] = 0;
-  __syncthreads();
+  // a sub-cell of the set is known to be too full: the build will be redone
+  if (__syncthreads_or(threadIdx.x == 0 && ld_relaxed_u32(S.info + 2) != 0)) return;
   const uint64_t base = (uint64_t)t * S.tile;
   const uint32_t cnt = (uint32_t)((S.n - base) < (uint64_t)S.tile ? (S.n - base) : S.tile);
   const float* xyz = S.xyz + 3 * base;
@@ -266,6 +274,7 @@ __global__ void __launch_bounds__(kScThreads, 1) bucket_scatter_kernel(
     for (int u = 0; u < 4; ++u) {
       const uint32_t c = c0 + u * kScThreads + threadIdx.x;
       if (hh[u]) s_at[c] = c * (uint32_t)kBkCap + r[u];
+      if (r[u] + hh[u] > (uint32_t)kBkCap) atomicExch(S.info + 2, 1u);
     }
   }
   __syncthreads();
@@ -407,7 +416,7 @@ __global__ void __launch_bounds__(kBkThreads, 3) bucket_boxes_kernel(
   uint64_t* B = reinterpret_cast<uint64_t*>(smem);          // the items, by group
   uint32_t* gs = reinterpret_cast<uint32_t*>(B + kBkCap);  // group counts, then starts [2^D + 1]
   uint16_t* ord = reinterpret_cast<uint16_t*>(gs + (1 << kBkGroupBits) + 4);  // sorted k: B[ord[k]]
-  __shared__ uint32_t s_t, s_abort;
+  __shared__ uint32_t s_abort;
   __shared__ uint64_t s_w[W + 1];
   __shared__ uint32_t s_R[kLevels], s_C[kLevels];
   __shared__ __align__(8) uint8_t s_fl[kBkHistCells];  // non-empty flags

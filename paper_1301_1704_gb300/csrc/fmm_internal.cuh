@@ -387,7 +387,8 @@ struct BkSet {
   uint32_t* sct;     // [8^(bl+1)] points per sub-cell (zeroed before the scatter)
   uint32_t* bcell;   // [nslot] non-empty cells, ascending
   uint32_t* boff;    // [nslot + 1] their bookmarks
-  uint32_t* info;    // [4]: non-empty cells, largest cell
+  uint32_t* info;    // [4]: non-empty cells, points of the fullest sub-cell (where one is too full),
+                     // whether a sub-cell is too full (zeroed)
   uint64_t* items;   // [8^(bl+1)][kBkCap] the points' items, sub-cell c's from slot c kBkCap
   uint32_t* soff;    // [8 * nslot] sub-cell bookmarks
   uint32_t* scnt;    // [8 * nslot] sub-cell sizes
