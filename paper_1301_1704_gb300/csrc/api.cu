@@ -25,6 +25,10 @@
 
 using namespace fmm;
 
+namespace fmm {
+thread_local bool capturing_thread = false;
+}
+
 namespace {
 
 struct Chunk {
@@ -127,7 +131,7 @@ int cap_begin(fmm_ctx* c) {
     c->graph_build = false;  // the rest of the build runs eagerly
     return FMM_OK;
   }
-  c->capturing = true;
+  c->capturing = capturing_thread = true;
   return FMM_OK;
 }
 
@@ -136,7 +140,7 @@ int cap_begin(fmm_ctx* c) {
 // shape changed) and is launched.
 int cap_end(fmm_ctx* c) {
   if (!c->capturing) return FMM_OK;
-  c->capturing = false;
+  c->capturing = capturing_thread = false;
   cudaGraph_t g = nullptr;
   if (cudaStreamEndCapture(c->stream, &g) != cudaSuccess || g == nullptr) {
     cudaGetLastError();
@@ -186,7 +190,7 @@ int cap_end(fmm_ctx* c) {
 void cap_abort(fmm_ctx* c) {
   c->graph_build = false;
   if (!c->capturing) return;
-  c->capturing = false;
+  c->capturing = capturing_thread = false;
   cudaGraph_t g = nullptr;
   cudaStreamEndCapture(c->stream, &g);
   if (g) cudaGraphDestroy(g);
@@ -340,6 +344,7 @@ struct Launch {
 // Zeroes up to two word ranges (16-byte aligned starts) in one launch.
 __global__ void __launch_bounds__(256) zero_words_kernel(uint32_t* __restrict__ p0, uint64_t w0,
                                                          uint32_t* __restrict__ p1, uint64_t w1) {
+  grid_wait();
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   const uint64_t t0 = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
 #pragma unroll
@@ -356,6 +361,7 @@ __global__ void __launch_bounds__(256) zero_words_kernel(uint32_t* __restrict__ 
 __global__ void __launch_bounds__(256) copy_words_kernel(const uint32_t* __restrict__ src,
                                                           uint32_t* __restrict__ dst,
                                                           uint64_t words) {
+  grid_wait(src);
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < words; i += stride)
     dst[i] = src[i];
@@ -375,7 +381,7 @@ int dev_zero2(fmm_ctx* c, void* p0, size_t b0, void* p1, size_t b1) {
     return FMM_ERR_ARG;
   Launch L(c, "zero");
   const uint64_t w0 = b0 / 4, w1 = b1 / 4;
-  zero_words_kernel<<<small_grid(std::max(w0, w1) / 4), 256, 0, c->stream>>>(
+  launch_k(zero_words_kernel, small_grid(std::max(w0, w1) / 4), 256, 0, c->stream, 
       static_cast<uint32_t*>(p0), w0, static_cast<uint32_t*>(p1), w1);
   return cudaGetLastError() == cudaSuccess ? FMM_OK : FMM_ERR_CUDA;
 }
@@ -560,7 +566,7 @@ char* upload(fmm_ctx* c, const Upload& up, int* err) {
   {
     Launch L(c, "upload");
     const uint64_t words = (need + 3) / 4;  // the staging buffer and the arena block hold the rounding
-    copy_words_kernel<<<small_grid(words), 256, 0, c->stream>>>(static_cast<const uint32_t*>(hd),
+    launch_k(copy_words_kernel, small_grid(words), 256, 0, c->stream, static_cast<const uint32_t*>(hd),
                                                                  reinterpret_cast<uint32_t*>(dev),
                                                                  words);
   }

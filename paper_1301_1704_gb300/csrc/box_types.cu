@@ -27,6 +27,7 @@ namespace {
 __global__ void __launch_bounds__(256) on_node_kernel(const uint32_t* __restrict__ owner,
                                                       uint32_t nbox, uint32_t node,
                                                       uint8_t* __restrict__ on) {
+  grid_wait(owner);
   for (uint32_t b = blockIdx.x * blockDim.x + threadIdx.x; b < nbox; b += gridDim.x * blockDim.x)
     on[b] = owner[b] == node;
 }
@@ -37,6 +38,7 @@ __global__ void __launch_bounds__(256) on_node_kernel(const uint32_t* __restrict
 __global__ void __launch_bounds__(256) child_sides_kernel(const uint32_t* __restrict__ child,
                                                           const uint8_t* __restrict__ on_par,
                                                           uint32_t nbox, uint8_t* __restrict__ sides) {
+  grid_wait(child, on_par);
   for (uint32_t b = blockIdx.x * blockDim.x + threadIdx.x; b < nbox; b += gridDim.x * blockDim.x) {
     uint32_t s = 0;
     if (!child)
@@ -83,6 +85,7 @@ struct TypeArgs {
 };
 
 __global__ void __launch_bounds__(256) box_type_kernel(TypeArgs g, uint32_t nbox, int mode) {
+  grid_wait();
   const uint32_t l8 = threadIdx.x & 7u;
   const uint32_t g0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 3, groups = (gridDim.x * blockDim.x) >> 3;
   for (uint32_t w0 = g0 & ~3u; w0 < nbox; w0 += groups) {  // (the same rounds for a whole warp)
@@ -141,13 +144,13 @@ uint32_t grid_for(uint32_t n) {
 void launch_on_node(const uint32_t* owner, uint32_t nbox, uint32_t node, uint8_t* on,
                     cudaStream_t s) {
   if (nbox == 0) return;
-  on_node_kernel<<<grid_for(nbox), 256, 0, s>>>(owner, nbox, node, on);
+  launch_k(on_node_kernel, grid_for(nbox), 256, 0, s, owner, nbox, node, on);
 }
 
 void launch_child_sides(const uint32_t* child, const uint8_t* on_par, uint32_t nbox,
                         uint8_t* sides, cudaStream_t s) {
   if (nbox == 0) return;
-  child_sides_kernel<<<grid_for(nbox), 256, 0, s>>>(child, on_par, nbox, sides);
+  launch_k(child_sides_kernel, grid_for(nbox), 256, 0, s, child, on_par, nbox, sides);
 }
 
 void launch_box_type(const fmm_tree& t, int l, int mode, const uint8_t* side, const uint8_t* on,
@@ -159,7 +162,7 @@ void launch_box_type(const fmm_tree& t, int l, int mode, const uint8_t* side, co
              on_next ? t.child_src[l] : nullptr, side, on, border_up, border, on_next, type};
   uint32_t grid = (nbox + 31) / 32;  // 32 boxes a block
   if (grid > 152u * 8u) grid = 152u * 8u;
-  box_type_kernel<<<grid, 256, 0, s>>>(g, nbox, mode);
+  launch_k(box_type_kernel, grid, 256, 0, s, g, nbox, mode);
 }
 
 }  // namespace fmm

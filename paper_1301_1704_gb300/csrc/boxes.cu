@@ -50,6 +50,7 @@ __global__ void __launch_bounds__(kBoxThreads) finish_boxes_kernel(const Seg* __
   uint8_t* s_dd = reinterpret_cast<uint8_t*>(s_key) + kBoxDdOff;  // first differing level
   uint32_t* s_val = reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(s_key) + kBoxValOff);
 
+  grid_wait(segs, slots);
   const Seg& sg = segs[slots[find_slot(slots, nslots, blockIdx.x)].seg];
   const uint64_t* __restrict__ keys = sg.skeys;
   const uint32_t* __restrict__ vals = sg.svals;
@@ -252,6 +253,7 @@ __global__ void __launch_bounds__(kBoxThreads, NL <= 8 ? 4 : 1) coarse_boxes_ker
   __shared__ uint32_t s_texcl[kLevels];
   __shared__ uint32_t s_ttot[kLevels];
   __shared__ uint64_t s_key[kBoxTile + 1];  // s_key[j + 1] = level-Lb key of box t0 + j
+  grid_wait(segs, slots);
   const Seg& sg = segs[slots[find_slot(slots, nslots, blockIdx.x)].seg];
   const int Lb = sg.Lb;
   const LevelArrays& lv = sg.lv;
@@ -390,20 +392,20 @@ void launch_finish_boxes(const Seg* segs, const Slot* slots, uint32_t nslots, ui
     return true;
   }();
   (void)attr;
-  finish_boxes_kernel<<<units, kBoxThreads, kBoxSmem, s>>>(segs, slots, nslots, st, wait_ns);
+  launch_k(finish_boxes_kernel, units, kBoxThreads, kBoxSmem, s, segs, slots, nslots, st, wait_ns);
 }
 
 void launch_coarse_boxes(const Seg* segs, const Slot* slots, uint32_t nslots, uint32_t units,
                          int max_lb, DevStatus* st, uint64_t wait_ns, cudaStream_t s) {
   if (units == 0) return;
   if (max_lb <= 8)
-    coarse_boxes_kernel<8><<<units, kBoxThreads, 0, s>>>(segs, slots, nslots, st, wait_ns);
+    launch_k(coarse_boxes_kernel<8>, units, kBoxThreads, 0, s, segs, slots, nslots, st, wait_ns);
   else if (max_lb <= 12)
-    coarse_boxes_kernel<12><<<units, kBoxThreads, 0, s>>>(segs, slots, nslots, st, wait_ns);
+    launch_k(coarse_boxes_kernel<12>, units, kBoxThreads, 0, s, segs, slots, nslots, st, wait_ns);
   else if (max_lb <= 16)
-    coarse_boxes_kernel<16><<<units, kBoxThreads, 0, s>>>(segs, slots, nslots, st, wait_ns);
+    launch_k(coarse_boxes_kernel<16>, units, kBoxThreads, 0, s, segs, slots, nslots, st, wait_ns);
   else
-    coarse_boxes_kernel<kLevels><<<units, kBoxThreads, 0, s>>>(segs, slots, nslots, st, wait_ns);
+    launch_k(coarse_boxes_kernel<kLevels>, units, kBoxThreads, 0, s, segs, slots, nslots, st, wait_ns);
 }
 
 // ---------------------------------------------------------------------------
@@ -416,6 +418,7 @@ __global__ void __launch_bounds__(256) occupancy_kernel(const Seg* __restrict__ 
                                                         const Slot* __restrict__ slots,
                                                         uint32_t nslots, uint32_t unit_first,
                                                         const DevStatus* st) {
+  grid_wait(segs, slots);
   if (failed(st)) return;
   const uint32_t unit = blockIdx.x + unit_first;
   const uint32_t k = find_slot(slots, nslots, unit);
@@ -439,7 +442,7 @@ __global__ void __launch_bounds__(256) occupancy_kernel(const Seg* __restrict__ 
 void launch_occupancy(const Seg* segs, const Slot* slots, uint32_t nslots, uint32_t units,
                       uint32_t unit_first, DevStatus* st, cudaStream_t s) {
   if (units == 0) return;
-  occupancy_kernel<<<units, 256, 0, s>>>(segs, slots, nslots, unit_first, st);
+  launch_k(occupancy_kernel, units, 256, 0, s, segs, slots, nslots, unit_first, st);
 }
 
 uint32_t occupancy_units(uint32_t n) { return 1u + n / 16384u; }
@@ -458,6 +461,7 @@ __global__ void __launch_bounds__(256) depth_kernel(const Seg* __restrict__ segs
                                                     uint32_t nslots, uint32_t s,
                                                     uint32_t* __restrict__ out,
                                                     const DevStatus* st) {
+  grid_wait(segs, slots);
   if (failed(st)) return;
   const uint32_t k = find_slot(slots, nslots, blockIdx.x);
   const uint32_t set = slots[k].seg;
@@ -483,7 +487,7 @@ __global__ void __launch_bounds__(256) depth_kernel(const Seg* __restrict__ segs
 void launch_depth(const Seg* segs, const Slot* slots, uint32_t nslots, uint32_t units, uint32_t s,
                   uint32_t* out, DevStatus* st, cudaStream_t stream) {
   if (units == 0) return;
-  depth_kernel<<<units, 256, 0, stream>>>(segs, slots, nslots, s, out, st);
+  launch_k(depth_kernel, units, 256, 0, stream, segs, slots, nslots, s, out, st);
 }
 
 }  // namespace fmm

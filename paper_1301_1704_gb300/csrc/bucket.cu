@@ -102,6 +102,7 @@ __global__ void __launch_bounds__(kBkPlanThreads) bucket_plan_kernel(const BkSet
   constexpr int kPer = kBkMaxCells / kBkPlanThreads;  // cells per thread, at most
   __shared__ uint64_t s_w[W];
   __shared__ uint32_t s_max[W];
+  grid_wait(bsets);
   if (failed(st)) return;
   const BkSet& S = bsets[blockIdx.x];
   const uint32_t cells = bk_cells(S.bl);
@@ -208,6 +209,7 @@ __global__ void __launch_bounds__(kScThreads, 1) bucket_scatter_kernel(
     const BkSet* __restrict__ bsets, const Slot* __restrict__ slots, uint32_t nslots,
     uint32_t t_first, DevStatus* st) {
   extern __shared__ uint32_t s_at[];  // per sub-cell: the tile's count, then its next slot
+  grid_wait(bsets, slots);
   if (failed(st)) return;
   const uint32_t unit = blockIdx.x + t_first;  // (a launch may start past unit 0)
   const Slot sl = slots[find_slot(slots, nslots, unit)];
@@ -427,6 +429,7 @@ __global__ void __launch_bounds__(kBkThreads, 3) bucket_boxes_kernel(
   __shared__ BoxJob S;
 
   const int tid = threadIdx.x, lane = tid & 31;
+  grid_wait(bsets, segs, slots);
   if (tid == 0) {
     s_abort = failed(st) ? 1u : 0u;
     S.more = 0;
@@ -743,7 +746,7 @@ __global__ void __launch_bounds__(kBkThreads, 3) bucket_boxes_kernel(
 // ---------------------------------------------------------------------------
 void launch_bucket_plan(const BkSet* bsets, uint32_t nsets, DevStatus* st, cudaStream_t s) {
   if (nsets == 0) return;
-  bucket_plan_kernel<<<nsets, kBkPlanThreads, 0, s>>>(bsets, st);
+  launch_k(bucket_plan_kernel, nsets, kBkPlanThreads, 0, s, bsets, st);
 }
 
 void launch_bucket_scatter(const BkSet* bsets, const Slot* slots, uint32_t nslots, uint32_t t_first,
@@ -756,7 +759,7 @@ void launch_bucket_scatter(const BkSet* bsets, const Slot* slots, uint32_t nslot
   }();
   (void)attr;
   const size_t smem = sizeof(uint32_t) * 8 * (1u << (3 * max_bl));
-  bucket_scatter_kernel<<<tiles, kScThreads, smem, s>>>(bsets, slots, nslots, t_first, st);
+  launch_k(bucket_scatter_kernel, tiles, kScThreads, smem, s, bsets, slots, nslots, t_first, st);
 }
 
 void launch_bucket_boxes(const BkSet* bsets, const Seg* segs, const Slot* slots, uint32_t nslots,
@@ -770,7 +773,7 @@ void launch_bucket_boxes(const BkSet* bsets, const Seg* segs, const Slot* slots,
     return true;
   }();
   (void)attr;
-  bucket_boxes_kernel<<<units * 8, kBkThreads, kBkSmem, s>>>(bsets, segs, slots, nslots, ticket, st,
+  launch_k(bucket_boxes_kernel, units * 8, kBkThreads, kBkSmem, s, bsets, segs, slots, nslots, ticket, st,
                                                              wait_ns);
 }
 

@@ -25,6 +25,7 @@ __global__ void __launch_bounds__(256) fg_count_kernel(const Seg* __restrict__ s
                                                        uint64_t* __restrict__ keys_out,
                                                        uint32_t* __restrict__ ranks_out,
                                                        DevStatus* st) {
+  grid_wait(segs, slots);
   const Slot sl = slots[find_slot(slots, nslots, blockIdx.x)];
   const Seg& sg = segs[sl.seg];
   const uint64_t base = (uint64_t)(blockIdx.x - sl.unit0) * sg.tile;
@@ -58,6 +59,7 @@ __global__ void __launch_bounds__(256) fg_move_kernel(const Seg* __restrict__ se
                                                       uint64_t* __restrict__ keys_out,
                                                       uint32_t* __restrict__ vals_out,
                                                       const DevStatus* st) {
+  grid_wait(segs, slots);
   if (failed(st)) return;
   const Slot sl = slots[find_slot(slots, nslots, blockIdx.x)];
   const Seg& sg = segs[sl.seg];
@@ -84,14 +86,14 @@ void launch_fg_count(const Seg* segs, const Slot* slots, uint32_t nslots, uint32
                      uint32_t* bins, uint64_t* keys_out, uint32_t* ranks_out, DevStatus* st,
                      cudaStream_t s) {
   if (ntiles == 0) return;
-  fg_count_kernel<<<ntiles, 256, 0, s>>>(segs, slots, nslots, bins, keys_out, ranks_out, st);
+  launch_k(fg_count_kernel, ntiles, 256, 0, s, segs, slots, nslots, bins, keys_out, ranks_out, st);
 }
 
 void launch_fg_move(const Seg* segs, const Slot* slots, uint32_t nslots, uint32_t ntiles,
                     const uint32_t* bins, const uint64_t* keys_in, const uint32_t* ranks_in,
                     uint64_t* keys_out, uint32_t* vals_out, DevStatus* st, cudaStream_t s) {
   if (ntiles == 0) return;
-  fg_move_kernel<<<ntiles, 256, 0, s>>>(segs, slots, nslots, bins, keys_in, ranks_in, keys_out,
+  launch_k(fg_move_kernel, ntiles, 256, 0, s, segs, slots, nslots, bins, keys_in, ranks_in, keys_out,
                                         vals_out, st);
 }
 

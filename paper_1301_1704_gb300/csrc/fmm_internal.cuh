@@ -84,6 +84,49 @@ __device__ __forceinline__ uint64_t morton_key(float x, float y, float z, bool* 
 }
 
 // ---------------------------------------------------------------------------
+// Programmatic dependent launch.  A build is a chain of short kernels on one
+// stream; launched by launch_k, a kernel's blocks are placed while the kernel
+// before it drains, and wait here for its end and its writes.  Every kernel that
+// launch_k launches calls grid_wait before it reads or writes anything but its
+// parameters and shared memory -- then a kernel's end implies the ends of all
+// before it -- and lets the next kernel's blocks come once that wait is over.
+// The pointers advance by a zero that the wait makes, so that no load through
+// them is moved above it (and they stay the parameters' for alias analysis).
+template <class... P>
+__device__ __forceinline__ void grid_wait(P&... p) {
+  uint32_t zero;
+  asm volatile("griddepcontrol.wait;\n\tmov.u32 %0, 0;" : "=r"(zero)::"memory");
+  ((p += zero), ...);
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// Only grids of up to two blocks an SM come early: a large kernel's blocks would
+// wait beside a large kernel's for its whole run (512 sets in one build: 8.65 ms
+// so, 8.88 to 9.3 ms with every kernel early) and have little to gain.  16384
+// points 147 -> 122 us, 24 small sets 435 -> 374, 300001/200003 points 332 -> 274,
+// cluster size of 10^6 points 783 -> 706.  Nor do kernels recorded into a graph:
+// recording and updating programmatic edges costs the host what they save
+// (10^6-point time step in graph mode: 515 us, 530 with them).
+constexpr uint32_t kEarlyGrid = 152u * 2u;
+extern thread_local bool capturing_thread;  // this thread records its launches (api.cu)
+
+template <class... K, class... A>
+inline void launch_k(void (*kernel)(K...), uint32_t grid, uint32_t block, size_t smem,
+                     cudaStream_t s, A... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = grid <= kEarlyGrid && !capturing_thread ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<K>(args)...);
+}
+
+// ---------------------------------------------------------------------------
 // Decoupled look-back words: 2 flag bits over a 62-bit value.
 constexpr uint64_t kFlagAgg = 1ull << 62;
 constexpr uint64_t kFlagIncl = 2ull << 62;

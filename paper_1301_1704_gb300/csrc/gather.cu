@@ -12,6 +12,7 @@ namespace {
 __global__ void __launch_bounds__(256) sorted_xyz_kernel(const Seg* __restrict__ segs,
                                                          const Slot* __restrict__ slots,
                                                          uint32_t nslots, const DevStatus* st) {
+  grid_wait(segs, slots);
   if (failed(st)) return;
   const Slot sl = slots[find_slot(slots, nslots, blockIdx.x)];
   const Seg& sg = segs[sl.seg];
@@ -35,6 +36,7 @@ __global__ void __launch_bounds__(256) e2_count_kernel(const uint32_t* __restric
                                                        const uint32_t* __restrict__ src_off,
                                                        uint32_t nrecv, uint32_t* __restrict__ out,
                                                        DevStatus* st) {
+  grid_wait(e2_off, e2_idx, src_off);
   for (uint32_t r = blockIdx.x * blockDim.x + threadIdx.x; r < nrecv;
        r += gridDim.x * blockDim.x) {
     uint64_t c = 0;
@@ -60,6 +62,7 @@ __global__ void __launch_bounds__(256) e2_gather_kernel(const uint32_t* __restri
                                                         const float* __restrict__ sorted_src,
                                                         const uint32_t* __restrict__ off,
                                                         uint32_t nrecv, float* __restrict__ out) {
+  grid_wait(e2_off, off);
   const uint32_t lane = threadIdx.x & 31;
   const uint32_t below = lanemask_lt() | (1u << lane);
   const uint32_t nw = (gridDim.x * blockDim.x) >> 5;
@@ -113,6 +116,7 @@ __global__ void __launch_bounds__(256) e2_gather_kernel(const uint32_t* __restri
 __global__ void __launch_bounds__(256) sorted_xyz_one_kernel(const uint32_t* __restrict__ perm,
                                                              const float* __restrict__ xyz,
                                                              uint32_t n, float* __restrict__ out) {
+  grid_wait(perm);
   for (uint64_t j = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; j < n;
        j += (uint64_t)gridDim.x * blockDim.x) {
     const uint64_t i = perm[j];
@@ -130,13 +134,13 @@ void launch_sorted_xyz_one(const uint32_t* perm, const float* xyz, uint32_t n, f
   if (n == 0) return;
   uint32_t grid = (n + 255) / 256;
   if (grid > 152u * 8u) grid = 152u * 8u;
-  sorted_xyz_one_kernel<<<grid, 256, 0, s>>>(perm, xyz, n, out);
+  launch_k(sorted_xyz_one_kernel, grid, 256, 0, s, perm, xyz, n, out);
 }
 
 void launch_sorted_xyz(const Seg* segs, const Slot* slots, uint32_t nslots, uint32_t units,
                        DevStatus* st, cudaStream_t s) {
   if (units == 0) return;
-  sorted_xyz_kernel<<<units, 256, 0, s>>>(segs, slots, nslots, st);
+  launch_k(sorted_xyz_kernel, units, 256, 0, s, segs, slots, nslots, st);
 }
 
 void launch_e2_count(const uint32_t* e2_off, const uint32_t* e2_idx, const uint32_t* src_off,
@@ -144,7 +148,7 @@ void launch_e2_count(const uint32_t* e2_off, const uint32_t* e2_idx, const uint3
   if (nrecv == 0) return;
   uint32_t grid = (nrecv + 255) / 256;
   if (grid > 152u * 8u) grid = 152u * 8u;
-  e2_count_kernel<<<grid, 256, 0, s>>>(e2_off, e2_idx, src_off, nrecv, out, st);
+  launch_k(e2_count_kernel, grid, 256, 0, s, e2_off, e2_idx, src_off, nrecv, out, st);
 }
 
 void launch_e2_gather(const uint32_t* e2_off, const uint32_t* e2_idx, const uint32_t* src_off,
@@ -153,7 +157,7 @@ void launch_e2_gather(const uint32_t* e2_off, const uint32_t* e2_idx, const uint
   if (nrecv == 0) return;
   uint32_t grid = (nrecv + 7) / 8;  // 8 warps a block
   if (grid > 152u * 16u) grid = 152u * 16u;
-  e2_gather_kernel<<<grid, 256, 0, s>>>(e2_off, e2_idx, src_off, sorted_src, off, nrecv, out);
+  launch_k(e2_gather_kernel, grid, 256, 0, s, e2_off, e2_idx, src_off, sorted_src, off, nrecv, out);
 }
 
 }  // namespace fmm

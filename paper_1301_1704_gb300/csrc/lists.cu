@@ -134,6 +134,7 @@ __global__ void __launch_bounds__(1024) list_plan_kernel(const Seg* __restrict__
                                                          uint32_t njobs, const ListLevel* lvls,
                                                          const DevStatus* st) {
   __shared__ uint32_t s_sum[33];
+  grid_wait(segs, jobs);
   if (failed(st)) return;
   const int l = 2 + blockIdx.x;
   const ListLevel& LV = lvls[l];
@@ -161,7 +162,7 @@ __global__ void __launch_bounds__(1024) list_plan_kernel(const Seg* __restrict__
 void launch_list_plan(const Seg* segs, const Job* jobs, uint32_t njobs, int Lmax,
                       const ListLevel* lvls, DevStatus* st, cudaStream_t s) {
   if (njobs <= 1 || Lmax < 2) return;  // one job: its chunks follow from its box counts
-  list_plan_kernel<<<(uint32_t)(Lmax - 1), 1024, 0, s>>>(segs, jobs, njobs, lvls, st);
+  launch_k(list_plan_kernel, (uint32_t)(Lmax - 1), 1024, 0, s, segs, jobs, njobs, lvls, st);
 }
 
 // Job whose chunks hold chunk c: jc[j] <= c < jc[j + 1].
@@ -240,15 +241,16 @@ __global__ void __launch_bounds__(kListThreads, 6) list_count_kernel(
   __shared__ WarpJob s_job[kCountWarps];
   __shared__ uint64_t s_sum[2][kCountWarps + 1];
   __shared__ uint32_t s_last;
-  if (failed(st)) return;  // set before this launch: the same for every thread
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (tid < kNbor) s_mask[tid] = code_masks(tid);
+  grid_wait(segs, jobs);
+  if (failed(st)) return;  // set before this launch: the same for every thread
   const int sub = lane >> 3, l8 = lane & 7;
   const uint32_t chunks = njobs == 1 ? job_chunks(jobs[0], segs, l) : LV.jchunks[njobs];
   const uint32_t passes = count_passes(chunks), range = count_range(chunks);
   const uint32_t b0 = blockIdx.x * range;
   const uint32_t nblocks = range ? (chunks + range - 1) / range : 0u;
   if (blockIdx.x >= max(nblocks, 1u)) return;
-  if (tid < kNbor) s_mask[tid] = code_masks(tid);
   __syncthreads();
   WarpJob& W = s_job[warp];
   uint32_t jend = 0;
@@ -638,13 +640,7 @@ __global__ void __launch_bounds__(kListThreads, 4) list_fill_kernel(
   extern __shared__ __align__(16) unsigned char smem_raw[];
   FillSmem& sm = *reinterpret_cast<FillSmem*>(smem_raw);
   __shared__ WarpJob s_job[kFillWarps];
-  if (failed(st)) return;  // set before this launch: the same for every thread
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const uint32_t chunks = njobs == 1 ? job_chunks(jobs[0], segs, l) : LV.jchunks[njobs];
-  // A warp takes whole chunks, or in small levels a part of one.
-  const uint32_t warps = gridDim.x * kFillWarps;
-  const uint32_t split = 4u * chunks <= warps ? 4u : (2u * chunks <= warps ? 2u : 1u);
-  if (blockIdx.x * kFillWarps >= chunks * split) return;
   if (tid < kNbor) sm.mask[tid] = code_masks(tid);
   for (int t = tid; t < 256; t += kListThreads) {
     uint32_t sel = 0, n = 0;
@@ -652,6 +648,13 @@ __global__ void __launch_bounds__(kListThreads, 4) list_fill_kernel(
       if ((t >> rho) & 1) sel |= rho << (4 * n++);
     sm.sel[t] = sel;
   }
+  grid_wait(segs, jobs);
+  if (failed(st)) return;  // set before this launch: the same for every thread
+  const uint32_t chunks = njobs == 1 ? job_chunks(jobs[0], segs, l) : LV.jchunks[njobs];
+  // A warp takes whole chunks, or in small levels a part of one.
+  const uint32_t warps = gridDim.x * kFillWarps;
+  const uint32_t split = 4u * chunks <= warps ? 4u : (2u * chunks <= warps ? 2u : 1u);
+  if (blockIdx.x * kFillWarps >= chunks * split) return;
   __syncthreads();
   const uint32_t range = count_range(chunks);
   FillWarp& F = sm.w[warp];
@@ -761,7 +764,7 @@ void launch_list_count(const Seg* segs, const Job* jobs, uint32_t njobs, int l,
                        const ListLevel& lv, const ListLevel& up, uint32_t max_chunks, DevStatus* st,
                        cudaStream_t s) {
   const uint32_t grid = std::min((max_chunks + kCountWarps - 1) / kCountWarps, kCountGrid);
-  list_count_kernel<<<std::max(grid, 1u), kListThreads, 0, s>>>(segs, jobs, njobs, l, lv, up, st);
+  launch_k(list_count_kernel, std::max(grid, 1u), kListThreads, 0, s, segs, jobs, njobs, l, lv, up, st);
 }
 
 void launch_list_fill(const Seg* segs, const Job* jobs, uint32_t njobs, int l,
@@ -779,9 +782,9 @@ void launch_list_fill(const Seg* segs, const Job* jobs, uint32_t njobs, int l,
   const uint32_t grid = (uint32_t)std::max<uint64_t>(
       std::min<uint64_t>((units + kFillWarps - 1) / kFillWarps, kFillGrid), 1u);
   if (lv.code2)
-    list_fill_kernel<true><<<grid, kListThreads, sizeof(FillSmem), s>>>(segs, jobs, njobs, l, lv, up, st);
+    launch_k(list_fill_kernel<true>, grid, kListThreads, sizeof(FillSmem), s, segs, jobs, njobs, l, lv, up, st);
   else
-    list_fill_kernel<false><<<grid, kListThreads, sizeof(FillSmem), s>>>(segs, jobs, njobs, l, lv, up, st);
+    launch_k(list_fill_kernel<false>, grid, kListThreads, sizeof(FillSmem), s, segs, jobs, njobs, l, lv, up, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -803,6 +806,7 @@ __global__ void __launch_bounds__(kScanThreads) scan_u32_kernel(uint32_t* data, 
   __shared__ uint32_t s_tile;
   __shared__ uint32_t s_wsum[W];
   __shared__ uint64_t s_prev;
+  grid_wait();
   const uint32_t count = (count_dev && *count_dev < cap) ? *count_dev : cap;
   const uint32_t need = scan_tiles_of(count);
   if (threadIdx.x == 0) s_tile = atomicAdd(counter, 1u);
@@ -897,7 +901,7 @@ __global__ void __launch_bounds__(kScanThreads) scan_u32_kernel(uint32_t* data, 
 void launch_scan_u32(uint32_t* data, const uint32_t* count_dev, uint32_t cap, uint64_t* status,
                      uint32_t* counter, uint64_t* total64, DevStatus* st, uint64_t wait_ns,
                      cudaStream_t s) {
-  scan_u32_kernel<<<scan_tiles(cap), kScanThreads, 0, s>>>(data, status, total64, count_dev, cap,
+  launch_k(scan_u32_kernel, scan_tiles(cap), kScanThreads, 0, s, data, status, total64, count_dev, cap,
                                                            counter, st, wait_ns);
 }
 

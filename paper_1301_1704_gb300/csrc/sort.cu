@@ -69,6 +69,7 @@ __global__ void __launch_bounds__(256) upfront_hist_kernel(const float* __restri
                                                            uint32_t* __restrict__ hist,
                                                            DevStatus* st) {
   __shared__ uint32_t sh[8 * kRadixMax];
+  grid_wait(xyz);
   for (int i = threadIdx.x; i < 8 * kRadixMax; i += blockDim.x) sh[i] = 0;
   __syncthreads();
   const uint32_t mask = (1u << bits) - 1u;
@@ -106,11 +107,12 @@ void launch_upfront_hist(const float* xyz, uint32_t n, const SortPlan& p, uint32
   uint32_t blocks = (uint32_t)(((uint64_t)n / 4 + 255) / 256);
   if (blocks > 152u * 8u) blocks = 152u * 8u;
   if (blocks == 0) blocks = 1;
-  upfront_hist_kernel<<<blocks, 256, 0, s>>>(xyz, n, p.passes, p.bits, p.lo, vec, hist, st);
+  launch_k(upfront_hist_kernel, blocks, 256, 0, s, xyz, n, p.passes, p.bits, p.lo, vec, hist, st);
 }
 
 // Exclusive scan of each pass's digit counts (one block, one warp per pass).
 __global__ void digit_scan_kernel(uint32_t* hist, int passes, int radix) {
+  grid_wait();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (warp >= passes) return;
   uint32_t* h = hist + warp * kRadixMax;
@@ -130,7 +132,7 @@ __global__ void digit_scan_kernel(uint32_t* hist, int passes, int radix) {
 
 void launch_digit_scan(const SortPlan& p, uint32_t* hist, cudaStream_t s) {
   if (p.passes == 0) return;
-  digit_scan_kernel<<<1, 32 * 8, 0, s>>>(hist, p.passes, 1 << p.bits);
+  launch_k(digit_scan_kernel, 1, 32 * 8, 0, s, hist, p.passes, 1 << p.bits);
 }
 
 // ---------------------------------------------------------------------------
@@ -156,6 +158,7 @@ __global__ void __launch_bounds__(kSortThreads, 2) onesweep_kernel(
 
   const uint32_t radix = 1u << bits, mask = radix - 1u;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  grid_wait(xyz, keys_in, vals_in, digit_base);
   for (int i = threadIdx.x; i < W * kRadixMax; i += kSortThreads) (&s_wcnt[0][0])[i] = 0;
   if (threadIdx.x == 0) {
     s_tile = atomicAdd(counter, 1u);
@@ -304,11 +307,11 @@ void launch_onesweep_pass(int pass, const float* xyz, const uint64_t* keys_in,
   (void)attr;
   const int shift = p.lo + pass * p.bits;
   if (pass == 0)
-    onesweep_kernel<true><<<p.ntiles, kSortThreads, kSortSmem, s>>>(
+    launch_k(onesweep_kernel<true>, p.ntiles, kSortThreads, kSortSmem, s, 
         xyz, nullptr, nullptr, keys_out, vals_out, n, shift, p.bits, digit_base, status, counter,
         st, wait_ns, stall_tile);
   else
-    onesweep_kernel<false><<<p.ntiles, kSortThreads, kSortSmem, s>>>(
+    launch_k(onesweep_kernel<false>, p.ntiles, kSortThreads, kSortSmem, s, 
         nullptr, keys_in, vals_in, keys_out, vals_out, n, shift, p.bits, digit_base, status,
         counter, st, wait_ns, -1);
 }
@@ -339,6 +342,7 @@ __global__ void __launch_bounds__(256) tile_hist_kernel(const Seg* __restrict__ 
                                                         DevStatus* st) {
   __shared__ uint32_t sh[kRadixMax];
   for (int i = threadIdx.x; i < kRadixMax; i += blockDim.x) sh[i] = 0;
+  grid_wait(segs, slots);
   const Slot sl = slots[find_slot(slots, nslots, blockIdx.x)];
   const Seg& sg = segs[sl.seg];
   const uint32_t t = blockIdx.x - sl.unit0;  // tile of the set
@@ -417,10 +421,10 @@ void launch_tile_hist(int pass, const Seg* segs, const Slot* slots, uint32_t nsl
                       TileRec* recs, DevStatus* st, cudaStream_t s) {
   if (ntiles == 0) return;
   if (pass == 0)
-    tile_hist_kernel<true><<<ntiles, 256, 0, s>>>(segs, slots, nslots, 0, nullptr, keys_out, hist,
+    launch_k(tile_hist_kernel<true>, ntiles, 256, 0, s, segs, slots, nslots, 0, nullptr, keys_out, hist,
                                                   recs, st);
   else
-    tile_hist_kernel<false><<<ntiles, 256, 0, s>>>(segs, slots, nslots, pass, keys, nullptr, hist,
+    launch_k(tile_hist_kernel<false>, ntiles, 256, 0, s, segs, slots, nslots, pass, keys, nullptr, hist,
                                                    recs, st);
 }
 
@@ -460,6 +464,7 @@ __global__ void __launch_bounds__(kSortThreads, ITEMS <= 7 ? 2 : 1) rts_scatter_
 
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t lt = lanemask_lt();
+  grid_wait(recs);
   if (threadIdx.x == 0) {
     s_fail = failed(st) ? 1u : 0u;
     mbar_init(&s_bar[0], 1);
@@ -669,13 +674,13 @@ void scatter_items(int pass, const TileRec* recs, uint32_t ntiles, const uint64_
   if (grid > ntiles) grid = ntiles;
   if (pass == 0) {
     if (stable)
-      rts_scatter_kernel<ITEMS, true, true><<<grid, kSortThreads, smem, s>>>(
+      launch_k(rts_scatter_kernel<ITEMS, true, true>, grid, kSortThreads, smem, s, 
           recs, ntiles, keys_in, nullptr, keys_out, vals_out, offsets, bulk, st, wait_ns);
     else
-      rts_scatter_kernel<ITEMS, true, false><<<grid, kSortThreads, smem, s>>>(
+      launch_k(rts_scatter_kernel<ITEMS, true, false>, grid, kSortThreads, smem, s, 
           recs, ntiles, keys_in, nullptr, keys_out, vals_out, offsets, bulk, st, wait_ns);
   } else {
-    rts_scatter_kernel<ITEMS, false, true><<<grid, kSortThreads, smem, s>>>(
+    launch_k(rts_scatter_kernel<ITEMS, false, true>, grid, kSortThreads, smem, s, 
         recs, ntiles, keys_in, vals_in, keys_out, vals_out, offsets, bulk, st, wait_ns);
   }
 }
