@@ -1306,12 +1306,13 @@ int run_build(fmm_ctx* c, std::vector<SetPlan>& sets, std::vector<JobPlan>& jobs
     launch_list_plan(m.segs, m.jobs, njobs, Lmax, m.lvls, c->st, s);
   }
   for (int l = 2; l <= Lmax; ++l) {
+    const LevelJob one = level_job(jobs[0].dev, sets[jobs[0].src].dev, sets[jobs[0].recv].dev, l, lvls[l - 1]);
     {
       Launch Lk(c, "list_count");
-      launch_list_count(m.segs, m.jobs, njobs, l, lvls[l], lvls[l - 1], chunks[l], c->st, s);
+      launch_list_count(m.segs, m.jobs, njobs, l, lvls[l], lvls[l - 1], one, chunks[l], c->st, s);
     }
     Launch Lk(c, "list_fill");
-    launch_list_fill(m.segs, m.jobs, njobs, l, lvls[l], lvls[l - 1], chunks[l], c->st, s);
+    launch_list_fill(m.segs, m.jobs, njobs, l, lvls[l], lvls[l - 1], one, chunks[l], c->st, s);
   }
   FMM_CUDA(cudaGetLastError());
 

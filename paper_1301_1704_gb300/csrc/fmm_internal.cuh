@@ -412,6 +412,26 @@ struct ListLevel {
   uint64_t* nnz;     // [njobs][2] E2 / E4 entries of each job (zeroed)
 };
 
+// What the list kernels read of a job at one level.  Builds of one job hand it to
+// the kernels as a parameter, where looking it up in the descriptors would put
+// five dependent loads before every small level's first useful one.
+struct LevelJob {
+  const uint32_t* off_up;   // E2 row starts, level l-1
+  const uint32_t* idx_up;   // E2 entries, level l-1
+  const uint8_t* code_up;   // ... and their offset codes
+  const uint32_t* rchild;   // receiver children, level l-1
+  const uint64_t* rkey;     // receiver keys, level l
+  const uint64_t* rkey1;    // ... and level 1
+  const uint8_t* socc;      // source child occupancy, level l-1
+  const uint32_t* schild;   // source children, level l-1
+  const uint64_t* skey1;    // source keys, level 1
+  const uint32_t* rnbox;    // receiver and source boxes per level
+  const uint32_t* snbox;
+  uint32_t* out2;           // row starts, level l
+  uint32_t* out4;
+  uint64_t slot;
+};
+
 // One point set on the bucket path (bucket.cu): the points are bucketed on
 // the sub-cells (level bl + 1) of the cells of level bl, in one pass, and
 // each sub-cell is sorted, and its boxes emitted, by one block.
@@ -576,18 +596,20 @@ uint32_t scan_tiles(uint32_t cap);
 
 // Lists of level l for every job, after one launch that plans the chunks of
 // every level (builds of several jobs; lvls: device array of kLevels
-// ListLevel).  lv, up: the host's copies of level l and of its parent level;
-// max_chunks: list_chunks of the level's parents.
+// ListLevel).  lv, up: the host's copies of level l and of its parent level; one:
+// level_job of a build's only job (unused where there are more); max_chunks:
+// list_chunks of the level's parents.
+LevelJob level_job(const Job& J, const Seg& src, const Seg& recv, int l, const ListLevel& up);
 uint32_t list_chunks(uint64_t cap, uint32_t njobs);
 uint32_t list_blocks();
 void launch_list_plan(const Seg* segs, const Job* jobs, uint32_t njobs, int Lmax,
                       const ListLevel* lvls, DevStatus* st, cudaStream_t s);
 void launch_list_count(const Seg* segs, const Job* jobs, uint32_t njobs, int l,
-                       const ListLevel& lv, const ListLevel& up, uint32_t max_chunks, DevStatus* st,
-                       cudaStream_t s);
+                       const ListLevel& lv, const ListLevel& up, const LevelJob& one,
+                       uint32_t max_chunks, DevStatus* st, cudaStream_t s);
 void launch_list_fill(const Seg* segs, const Job* jobs, uint32_t njobs, int l,
-                      const ListLevel& lv, const ListLevel& up, uint32_t max_chunks, DevStatus* st,
-                      cudaStream_t s);
+                      const ListLevel& lv, const ListLevel& up, const LevelJob& one,
+                      uint32_t max_chunks, DevStatus* st, cudaStream_t s);
 
 // Bucket path (bucket.cu).  count and scatter: units = tiles of the slots'
 // sets (slot seg = BkSet index); plan: one block per set; split: units =

@@ -179,42 +179,58 @@ __device__ __forceinline__ uint32_t find_job(const uint32_t* jc, uint32_t njobs,
 }
 
 // A warp's current job at level l.
-struct WarpJob {
-  const uint32_t* off_up;   // E2 row starts, level l-1
-  const uint32_t* idx_up;   // E2 entries, level l-1
-  const uint8_t* code_up;   // ... and their offset codes
-  const uint32_t* rchild;   // receiver children, level l-1
-  const uint64_t* rkey;     // receiver keys, level l
-  const uint8_t* socc;      // source child occupancy, level l-1
-  const uint32_t* schild;   // source children, level l-1
-  uint32_t* out2;           // row starts, level l
-  uint32_t* out4;
+struct WarpJob : LevelJob {
   uint64_t base2, base4;    // the level's entries before the job
   uint32_t j, chunk0, chunk1, np, nsrc1;
-  uint64_t slot;
 };
 
+__host__ __device__ inline LevelJob make_level_job(const Job& J, const Seg& S, const Seg& R, int l,
+                                                   const ListLevel& up) {
+  LevelJob v;
+  v.off_up = J.out2[l - 1];
+  v.idx_up = l > 2 ? up.idx2 + 27ull * J.slot[l - 1] : nullptr;
+  v.code_up = l > 2 ? up.code2 + 27ull * J.slot[l - 1] : nullptr;
+  v.rchild = R.lv.child[l - 1];
+  v.rkey = R.lv.key[l];
+  v.rkey1 = R.lv.key[1];
+  v.socc = S.lv.occ[l - 1];
+  v.schild = S.lv.child[l - 1];
+  v.skey1 = S.lv.key[1];
+  v.rnbox = R.nbox;
+  v.snbox = S.nbox;
+  v.out2 = J.out2[l];
+  v.out4 = J.out4[l];
+  v.slot = J.slot[l];
+  return v;
+}
+
+LevelJob level_job(const Job& J, const Seg& src, const Seg& recv, int l, const ListLevel& up) {
+  return make_level_job(J, src, recv, l, up);
+}
+
+// The job of chunk c (one lane).  one, np1: the only job and its parents, when
+// njobs = 1.
 __device__ void load_job(WarpJob& W, const Seg* segs, const Job* jobs, uint32_t njobs, int l,
-                         const ListLevel& LV, const ListLevel& up, uint32_t c) {
-  const uint32_t j = njobs == 1 ? 0u : find_job(LV.jchunks, njobs, c);
+                         const ListLevel& LV, const ListLevel& up, const LevelJob& one,
+                         uint32_t np1, uint32_t c) {
+  if (njobs == 1) {
+    static_cast<LevelJob&>(W) = one;
+    W.j = W.chunk0 = 0;
+    W.np = np1;
+    W.chunk1 = (np1 + kChunk - 1) / kChunk;
+    W.nsrc1 = l == 2 ? min(one.snbox[1], 8u) : 0u;
+    return;
+  }
+  const uint32_t j = find_job(LV.jchunks, njobs, c);
   const Job& J = jobs[j];
-  const Seg& S = segs[J.src];
-  const Seg& R = segs[J.recv];
+  const LevelJob v = make_level_job(J, segs[J.src], segs[J.recv], l, up);
+  const uint32_t np = v.rnbox[l - 1], ns = v.snbox[1], c0 = LV.jchunks[j], c1 = LV.jchunks[j + 1];
+  static_cast<LevelJob&>(W) = v;
   W.j = j;
-  W.np = R.nbox[l - 1];
-  W.chunk0 = njobs == 1 ? 0u : LV.jchunks[j];
-  W.chunk1 = njobs == 1 ? (W.np + kChunk - 1) / kChunk : LV.jchunks[j + 1];
-  W.nsrc1 = min(S.nbox[1], 8u);
-  W.off_up = J.out2[l - 1];
-  W.idx_up = l > 2 ? up.idx2 + 27ull * J.slot[l - 1] : nullptr;
-  W.code_up = l > 2 ? up.code2 + 27ull * J.slot[l - 1] : nullptr;
-  W.rchild = R.lv.child[l - 1];
-  W.rkey = R.lv.key[l];
-  W.socc = S.lv.occ[l - 1];
-  W.schild = S.lv.child[l - 1];
-  W.out2 = J.out2[l];
-  W.out4 = J.out4[l];
-  W.slot = J.slot[l];
+  W.np = np;
+  W.chunk0 = c0;
+  W.chunk1 = c1;
+  W.nsrc1 = min(ns, 8u);
 }
 
 // At level 2 every pair of level-1 boxes touches: the offset code follows from
@@ -236,7 +252,8 @@ __device__ __forceinline__ uint32_t level1_code(uint32_t source, uint32_t receiv
 // box and a prefix sum launch a level.
 __global__ void __launch_bounds__(kListThreads, 6) list_count_kernel(
     const Seg* __restrict__ segs, const Job* __restrict__ jobs, uint32_t njobs, int l,
-    const __grid_constant__ ListLevel LV, const __grid_constant__ ListLevel up, DevStatus* st) {
+    const __grid_constant__ ListLevel LV, const __grid_constant__ ListLevel up,
+    const __grid_constant__ LevelJob one, DevStatus* st) {
   __shared__ uint2 s_mask[kNbor];
   __shared__ WarpJob s_job[kCountWarps];
   __shared__ uint64_t s_sum[2][kCountWarps + 1];
@@ -244,9 +261,10 @@ __global__ void __launch_bounds__(kListThreads, 6) list_count_kernel(
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (tid < kNbor) s_mask[tid] = code_masks(tid);
   grid_wait(segs, jobs);
-  if (failed(st)) return;  // set before this launch: the same for every thread
   const int sub = lane >> 3, l8 = lane & 7;
-  const uint32_t chunks = njobs == 1 ? job_chunks(jobs[0], segs, l) : LV.jchunks[njobs];
+  const uint32_t np1 = njobs == 1 ? one.rnbox[l - 1] : 0u;
+  const uint32_t chunks = njobs == 1 ? (np1 + kChunk - 1) / kChunk : LV.jchunks[njobs];
+  if (failed(st)) return;  // set before this launch: the same for every thread
   const uint32_t passes = count_passes(chunks), range = count_range(chunks);
   const uint32_t b0 = blockIdx.x * range;
   const uint32_t nblocks = range ? (chunks + range - 1) / range : 0u;
@@ -265,7 +283,7 @@ __global__ void __launch_bounds__(kListThreads, 6) list_count_kernel(
       if (c < b1) {
         if (c >= jend) {  // c only grows
           __syncwarp();
-          if (lane == 0) load_job(W, segs, jobs, njobs, l, LV, up, c);
+          if (lane == 0) load_job(W, segs, jobs, njobs, l, LV, up, one, np1, c);
           __syncwarp();
           jend = W.chunk1;
         }
@@ -290,8 +308,7 @@ __global__ void __launch_bounds__(kListThreads, 6) list_count_kernel(
           code[u] = 13;
           if (i < m) {
             if (l == 2) {
-              code[u] = level1_code((uint32_t)segs[jobs[W.j].src].lv.key[1][i],
-                                    (uint32_t)segs[jobs[W.j].recv].lv.key[1][p]);
+              code[u] = level1_code((uint32_t)W.skey1[i], (uint32_t)W.rkey1[p]);
             } else {
               q[u] = W.idx_up[first + i];
               code[u] = W.code_up[first + i];
@@ -393,18 +410,25 @@ __global__ void __launch_bounds__(kListThreads, 6) list_count_kernel(
     }
     __syncthreads();
   }
+  if (njobs == 1) {  // its totals are the level's
+    if (tid < 2) {
+      const uint64_t n = tot[tid];
+      LV.nnz[tid] = n;
+      (tid ? one.out4 : one.out2)[one.rnbox[l]] = (uint32_t)n;
+      if (n >> 32) set_error(st, FMM_ERR_CAPACITY);
+    }
+    return;
+  }
   for (uint32_t j = tid; j < njobs; j += kListThreads) {
     const Job& J = jobs[j];
     if (J.L < l) continue;
-    const uint32_t ca = njobs == 1 ? 0u : LV.jchunks[j];
-    const uint32_t cb = njobs == 1 ? chunks : LV.jchunks[j + 1];
     const auto entry = [&](uint32_t c, int d) -> uint64_t {
       if (c >= chunks) return tot[d];
       return LV.bbase[2 * (c / range) + d] + __ldcg((d ? LV.off4 : LV.off2) + (uint64_t)c * kChunk);
     };
     const uint32_t nrecv = segs[J.recv].nbox[l];
     for (int d = 0; d < 2; ++d) {
-      const uint64_t a = entry(ca, d), n = entry(cb, d) - a;
+      const uint64_t a = entry(LV.jchunks[j], d), n = entry(LV.jchunks[j + 1], d) - a;
       LV.jbase[2 * j + d] = a;
       LV.nnz[2 * j + d] = n;
       (d ? J.out4[l] : J.out2[l])[nrecv] = (uint32_t)n;
@@ -636,7 +660,8 @@ __device__ __forceinline__ void fill_parent(FillWarp& F, uint2 mk, uint32_t sel,
 template <bool kCodes>
 __global__ void __launch_bounds__(kListThreads, 4) list_fill_kernel(
     const Seg* __restrict__ segs, const Job* __restrict__ jobs, uint32_t njobs, int l,
-    const __grid_constant__ ListLevel LV, const __grid_constant__ ListLevel up, DevStatus* st) {
+    const __grid_constant__ ListLevel LV, const __grid_constant__ ListLevel up,
+    const __grid_constant__ LevelJob one, DevStatus* st) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   FillSmem& sm = *reinterpret_cast<FillSmem*>(smem_raw);
   __shared__ WarpJob s_job[kFillWarps];
@@ -649,8 +674,9 @@ __global__ void __launch_bounds__(kListThreads, 4) list_fill_kernel(
     sm.sel[t] = sel;
   }
   grid_wait(segs, jobs);
+  const uint32_t np1 = njobs == 1 ? one.rnbox[l - 1] : 0u;
+  const uint32_t chunks = njobs == 1 ? (np1 + kChunk - 1) / kChunk : LV.jchunks[njobs];
   if (failed(st)) return;  // set before this launch: the same for every thread
-  const uint32_t chunks = njobs == 1 ? job_chunks(jobs[0], segs, l) : LV.jchunks[njobs];
   // A warp takes whole chunks, or in small levels a part of one.
   const uint32_t warps = gridDim.x * kFillWarps;
   const uint32_t split = 4u * chunks <= warps ? 4u : (2u * chunks <= warps ? 2u : 1u);
@@ -664,9 +690,9 @@ __global__ void __launch_bounds__(kListThreads, 4) list_fill_kernel(
     const uint32_t c = u / split;  // (a power of two)
     if (c >= jend) {  // c only grows
       if (lane == 0) {
-        load_job(W, segs, jobs, njobs, l, LV, up, c);
-        W.base2 = LV.jbase[2 * W.j];
-        W.base4 = LV.jbase[2 * W.j + 1];
+        load_job(W, segs, jobs, njobs, l, LV, up, one, np1, c);
+        W.base2 = njobs == 1 ? 0ull : LV.jbase[2 * W.j];
+        W.base4 = njobs == 1 ? 0ull : LV.jbase[2 * W.j + 1];
       }
       __syncwarp();
       jend = W.chunk1;
@@ -704,9 +730,7 @@ __global__ void __launch_bounds__(kListThreads, 4) list_fill_kernel(
         cc[k] = 13u << 8;
         if (in[k]) {
           if (l == 2) {
-            cc[k] = level1_code((uint32_t)segs[jobs[W.j].src].lv.key[1][lane],
-                                (uint32_t)segs[jobs[W.j].recv].lv.key[1][p0 + k])
-                    << 8;
+            cc[k] = level1_code((uint32_t)W.skey1[lane], (uint32_t)W.rkey1[p0 + k]) << 8;
           } else {
             q[k] = W.idx_up[first + lane];
             cc[k] = (uint32_t)W.code_up[first + lane] << 8;
@@ -761,15 +785,16 @@ __global__ void __launch_bounds__(kListThreads, 4) list_fill_kernel(
 }
 
 void launch_list_count(const Seg* segs, const Job* jobs, uint32_t njobs, int l,
-                       const ListLevel& lv, const ListLevel& up, uint32_t max_chunks, DevStatus* st,
-                       cudaStream_t s) {
+                       const ListLevel& lv, const ListLevel& up, const LevelJob& one,
+                       uint32_t max_chunks, DevStatus* st, cudaStream_t s) {
   const uint32_t grid = std::min((max_chunks + kCountWarps - 1) / kCountWarps, kCountGrid);
-  launch_k(list_count_kernel, std::max(grid, 1u), kListThreads, 0, s, segs, jobs, njobs, l, lv, up, st);
+  launch_k(list_count_kernel, std::max(grid, 1u), kListThreads, 0, s, segs, jobs, njobs, l, lv, up, one,
+             st);
 }
 
 void launch_list_fill(const Seg* segs, const Job* jobs, uint32_t njobs, int l,
-                      const ListLevel& lv, const ListLevel& up, uint32_t max_chunks, DevStatus* st,
-                      cudaStream_t s) {
+                      const ListLevel& lv, const ListLevel& up, const LevelJob& one,
+                      uint32_t max_chunks, DevStatus* st, cudaStream_t s) {
   static const bool attr = [] {
     cudaFuncSetAttribute(list_fill_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)sizeof(FillSmem));
@@ -782,9 +807,11 @@ void launch_list_fill(const Seg* segs, const Job* jobs, uint32_t njobs, int l,
   const uint32_t grid = (uint32_t)std::max<uint64_t>(
       std::min<uint64_t>((units + kFillWarps - 1) / kFillWarps, kFillGrid), 1u);
   if (lv.code2)
-    launch_k(list_fill_kernel<true>, grid, kListThreads, sizeof(FillSmem), s, segs, jobs, njobs, l, lv, up, st);
+    launch_k(list_fill_kernel<true>, grid, kListThreads, sizeof(FillSmem), s, segs, jobs, njobs, l, lv, up, one,
+             st);
   else
-    launch_k(list_fill_kernel<false>, grid, kListThreads, sizeof(FillSmem), s, segs, jobs, njobs, l, lv, up, st);
+    launch_k(list_fill_kernel<false>, grid, kListThreads, sizeof(FillSmem), s, segs, jobs, njobs, l, lv, up, one,
+             st);
 }
 
 // ---------------------------------------------------------------------------
