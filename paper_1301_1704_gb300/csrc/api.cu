@@ -69,6 +69,7 @@ struct fmm_ctx {
   size_t cur = 0, off = 0;
   size_t peak_request = 0;
   DevStatus* st = nullptr;        // persistent device status word
+  bool st_stale = false;          // the next upload zeroes it
   void* up_buf = nullptr;         // pinned staging of descriptor uploads
   size_t up_bytes = 0, up_cursor = 0;
   void* rb_buf = nullptr;         // pinned read-back buffer
@@ -341,30 +342,38 @@ struct Launch {
 // Small transfers of a build done by the SMs, not the copy engines: on the
 // copy engines they would queue behind a large host copy of another set's
 // coordinates (a pipelined host-input build) and stall the stage they feed.
-// Zeroes up to two word ranges (16-byte aligned starts) in one launch.
-__global__ void __launch_bounds__(256) zero_words_kernel(uint32_t* __restrict__ p0, uint64_t w0,
-                                                         uint32_t* __restrict__ p1, uint64_t w1) {
+// Zeroes a word range (16-byte aligned start).
+__global__ void __launch_bounds__(256) zero_words_kernel(uint32_t* __restrict__ p, uint64_t words) {
   grid_wait();
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   const uint64_t t0 = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-#pragma unroll
-  for (int r = 0; r < 2; ++r) {
-    uint32_t* const p = r ? p1 : p0;
-    const uint64_t words = r ? w1 : w0;
-    const uint64_t n16 = words / 4;
-    uint4* q = reinterpret_cast<uint4*>(p);
-    for (uint64_t i = t0; i < n16; i += stride) q[i] = make_uint4(0u, 0u, 0u, 0u);
-    if (blockIdx.x == 0 && threadIdx.x < words - 4 * n16) p[4 * n16 + threadIdx.x] = 0u;
-  }
+  const uint64_t n16 = words / 4;
+  uint4* q = reinterpret_cast<uint4*>(p);
+  for (uint64_t i = t0; i < n16; i += stride) q[i] = make_uint4(0u, 0u, 0u, 0u);
+  if (blockIdx.x == 0 && threadIdx.x < words - 4 * n16) p[4 * n16 + threadIdx.x] = 0u;
 }
 
-__global__ void __launch_bounds__(256) copy_words_kernel(const uint32_t* __restrict__ src,
-                                                          uint32_t* __restrict__ dst,
-                                                          uint64_t words) {
+// Copies `words` and zeroes up to three word ranges (16-byte aligned starts) in one
+// launch: an upload of descriptors and the scratch its stage starts from.
+struct ZeroRange {
+  uint32_t* p;
+  uint64_t words;
+};
+__global__ void __launch_bounds__(256) copy_zero_kernel(const uint32_t* __restrict__ src,
+                                                         uint32_t* __restrict__ dst, uint64_t words,
+                                                         ZeroRange z0, ZeroRange z1, ZeroRange z2) {
   grid_wait(src);
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < words; i += stride)
-    dst[i] = src[i];
+  const uint64_t t0 = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
+  for (uint64_t i = t0; i < words; i += stride) dst[i] = src[i];
+#pragma unroll
+  for (int r = 0; r < 3; ++r) {
+    const ZeroRange z = r == 0 ? z0 : r == 1 ? z1 : z2;
+    const uint64_t n16 = z.words / 4;
+    uint4* q = reinterpret_cast<uint4*>(z.p);
+    for (uint64_t i = t0; i < n16; i += stride) q[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (blockIdx.x == 0 && threadIdx.x < z.words - 4 * n16) z.p[4 * n16 + threadIdx.x] = 0u;
+  }
 }
 
 uint32_t small_grid(uint64_t items) {
@@ -372,22 +381,15 @@ uint32_t small_grid(uint64_t items) {
   return (uint32_t)(g == 0 ? 1 : (g > 152u * 4u ? 152u * 4u : g));
 }
 
-// Zeroes [p0, p0 + b0) and [p1, p1 + b1) on the build's stream (16-byte
-// aligned starts, whole words).
-int dev_zero2(fmm_ctx* c, void* p0, size_t b0, void* p1, size_t b1) {
-  if (b0 == 0 && b1 == 0) return FMM_OK;
-  if (b0 % 4 != 0 || b1 % 4 != 0 || (reinterpret_cast<uintptr_t>(p0) & 15) != 0 ||
-      (reinterpret_cast<uintptr_t>(p1) & 15) != 0)
-    return FMM_ERR_ARG;
+// Zeroes `bytes` (a multiple of 4) at p (16-byte aligned) on the build's stream.
+int dev_zero(fmm_ctx* c, void* p, size_t bytes) {
+  if (bytes == 0) return FMM_OK;
+  if (bytes % 4 != 0 || (reinterpret_cast<uintptr_t>(p) & 15) != 0) return FMM_ERR_ARG;
   Launch L(c, "zero");
-  const uint64_t w0 = b0 / 4, w1 = b1 / 4;
-  launch_k(zero_words_kernel, small_grid(std::max(w0, w1) / 4), 256, 0, c->stream, 
-      static_cast<uint32_t*>(p0), w0, static_cast<uint32_t*>(p1), w1);
+  launch_k(zero_words_kernel, small_grid(bytes / 16), 256, 0, c->stream, static_cast<uint32_t*>(p),
+           bytes / 4);
   return cudaGetLastError() == cudaSuccess ? FMM_OK : FMM_ERR_CUDA;
 }
-
-// Zeroes `bytes` (a multiple of 4) at p (16-byte aligned).
-int dev_zero(fmm_ctx* c, void* p, size_t bytes) { return dev_zero2(c, p, bytes, nullptr, 0); }
 
 void collect_times(fmm_ctx* c) {
   for (auto& p : c->pending) {
@@ -538,9 +540,11 @@ struct Upload {
   }
 };
 
-// Copies `up` to fresh device memory on the build's stream; returns the
-// device address of its first byte.
-char* upload(fmm_ctx* c, const Upload& up, int* err) {
+// Copies `up` to fresh device memory on the build's stream and zeroes [z0, z0 + b0)
+// and [z1, z1 + b1) (16-byte aligned starts, whole words), and with a build's first
+// one its status word; returns the device address of the copy's first byte.
+char* upload(fmm_ctx* c, const Upload& up, int* err, void* z0 = nullptr, size_t b0 = 0,
+             void* z1 = nullptr, size_t b1 = 0) {
   const size_t need = up.bytes.size();
   char* dev = arena_get<char>(c, need + 256, err);
   if (*err) return nullptr;
@@ -566,9 +570,12 @@ char* upload(fmm_ctx* c, const Upload& up, int* err) {
   {
     Launch L(c, "upload");
     const uint64_t words = (need + 3) / 4;  // the staging buffer and the arena block hold the rounding
-    launch_k(copy_words_kernel, small_grid(words), 256, 0, c->stream, static_cast<const uint32_t*>(hd),
-                                                                 reinterpret_cast<uint32_t*>(dev),
-                                                                 words);
+    const ZeroRange r0{static_cast<uint32_t*>(z0), b0 / 4}, r1{static_cast<uint32_t*>(z1), b1 / 4};
+    const ZeroRange r2{reinterpret_cast<uint32_t*>(c->st), c->st_stale ? sizeof(DevStatus) / 4 : 0};
+    c->st_stale = false;
+    launch_k(copy_zero_kernel, small_grid(std::max({words, r0.words / 4, r1.words / 4})), 256, 0,
+             c->stream, static_cast<const uint32_t*>(hd), reinterpret_cast<uint32_t*>(dev), words, r0,
+             r1, r2);
   }
   if (cudaGetLastError() != cudaSuccess) {
     *err = FMM_ERR_CUDA;
@@ -727,7 +734,7 @@ int fixed_grid_sort(fmm_ctx* c, std::vector<SetPlan*>& sets, SortMem& m, uint64_
   for (size_t i = 0; i < sets.size(); ++i) segs_host[i] = sets[i]->dev;
   const size_t o_segs = up.add(segs_host.data(), segs_host.size());
   const size_t o_slots = up.add(slots.data(), slots.size());
-  char* dev = upload(c, up, &err);
+  char* dev = upload(c, up, &err, z, zb);
   if (err) return err;
   m.segs = reinterpret_cast<Seg*>(dev + o_segs);
   // the depth stage walks the sort's tiles through pass 0's slot table
@@ -735,7 +742,6 @@ int fixed_grid_sort(fmm_ctx* c, std::vector<SetPlan*>& sets, SortMem& m, uint64_
   m.pass_slots[0] = reinterpret_cast<Slot*>(dev + o_slots);
   m.pass_nslots[0] = (uint32_t)slots.size();
   m.pass_tiles[0] = tiles;
-  FMM_TRY(dev_zero(c, z, zb));
   {
     Launch L(c, "fg_count");
     launch_fg_count(m.segs, m.pass_slots[0], m.pass_nslots[0], tiles, bins, m.kb, m.vb, c->st, s);
@@ -835,12 +841,11 @@ int sort_sets(fmm_ctx* c, std::vector<SetPlan*>& sets, bool stall, uint64_t wait
   size_t o_pass[8] = {};
   for (int p = 0; p < m.max_passes; ++p)
     o_pass[p] = up.add(tab.slots[p].data(), tab.slots[p].size());
-  char* dev = upload(c, up, &err);
+  char* dev = upload(c, up, &err, zero, zero_bytes);
   if (err) return err;
   m.segs = reinterpret_cast<Seg*>(dev + o_segs);
   for (int p = 0; p < m.max_passes; ++p)
     m.pass_slots[p] = reinterpret_cast<Slot*>(dev + o_pass[p]);
-  FMM_TRY(dev_zero(c, zero, zero_bytes));
   return run_sort(c, sets, m, stall, wait_ns);
 }
 
@@ -992,13 +997,13 @@ int bucket_setup(fmm_ctx* c, std::vector<SetPlan>& sets, BucketMem* bm) {
   const size_t o_t = up.add(tile_slots.data(), tile_slots.size());
   const size_t o_o = up.add(one.data(), one.size());
   const size_t o_x = up.add(box_slots.data(), box_slots.size());
-  char* dev = upload(c, up, &err);
+  char* dev = upload(c, up, &err, zero, zero_bytes);
   if (err) return err;
   m.bsets = reinterpret_cast<BkSet*>(dev + o_b);
   m.tile_slots = reinterpret_cast<Slot*>(dev + o_t);
   m.one_slots = reinterpret_cast<Slot*>(dev + o_o);
   m.box_slots = reinterpret_cast<Slot*>(dev + o_x);
-  return dev_zero(c, zero, zero_bytes);
+  return FMM_OK;
 }
 
 // Scatter of tiles [t0, t1) of bucket set k (one-set slot {k, 0}), or of
@@ -1136,7 +1141,7 @@ int run_build(fmm_ctx* c, std::vector<SetPlan>& sets, std::vector<JobPlan>& jobs
 
   std::vector<ListLevel> lvls(kLevels);
   std::memset(lvls.data(), 0, sizeof(ListLevel) * kLevels);
-  auto upload_all = [&](bool with_lists) -> int {
+  auto upload_all = [&](bool with_lists, void* z0, size_t b0, void* z1, size_t b1) -> int {
     Upload up;
     std::vector<Seg> segs_host(nsets);
     for (uint32_t i = 0; i < nsets; ++i) segs_host[i] = sets[i].dev;
@@ -1152,7 +1157,7 @@ int run_build(fmm_ctx* c, std::vector<SetPlan>& sets, std::vector<JobPlan>& jobs
       o_jobs = up.add(jobs_host.data(), njobs);
       o_lvls = up.add(lvls.data(), kLevels);
     }
-    char* dev = upload(c, up, &err);
+    char* dev = upload(c, up, &err, z0, b0, z1, b1);
     if (err) return err;
     m.segs = reinterpret_cast<Seg*>(dev + o_segs);
     m.fin_slots = reinterpret_cast<Slot*>(dev + o_fin);
@@ -1221,9 +1226,8 @@ int run_build(fmm_ctx* c, std::vector<SetPlan>& sets, std::vector<JobPlan>& jobs
       for (int l = 2; l <= jp.L; ++l) jp.cap[l] = sets[jp.recv].cap[l];
     FMM_TRY(plan_lists());
   }
-  FMM_TRY(upload_all(async_lists));
-  FMM_TRY(dev_zero2(c, zero, zero_bytes, async_lists ? list_zero : nullptr,
-                    async_lists ? list_zero_bytes : 0));
+  FMM_TRY(upload_all(async_lists, zero, zero_bytes, async_lists ? list_zero : nullptr,
+                     async_lists ? list_zero_bytes : 0));
 
   if (early) {
     // a set's child occupancy needs only that set's boxes
@@ -1296,8 +1300,7 @@ int run_build(fmm_ctx* c, std::vector<SetPlan>& sets, std::vector<JobPlan>& jobs
     for (auto& jp : jobs)
       for (int l = 2; l <= jp.L; ++l) jp.cap[l] = rb->nbox[(size_t)jp.recv * kLevels + l];
     FMM_TRY(plan_lists());
-    FMM_TRY(upload_all(true));
-    FMM_TRY(dev_zero(c, list_zero, list_zero_bytes));
+    FMM_TRY(upload_all(true, list_zero, list_zero_bytes, nullptr, 0));
   }
 
   // ---- lists, levels 2..Lmax.
@@ -1453,7 +1456,7 @@ int do_builds_on(fmm_ctx* c, const PairIn* pairs, uint32_t npairs, const fmm_par
   c->up_cursor = 0;
   c->seg = 0;
   FMM_TRY(cap_begin(c));
-  FMM_TRY(dev_zero(c, c->st, sizeof(DevStatus)));
+  c->st_stale = true;
 
   // Sets (the same array given as a pair's sources and receivers is one set)
   // and jobs.
