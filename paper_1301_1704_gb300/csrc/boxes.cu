@@ -153,6 +153,21 @@ __global__ void __launch_bounds__(kBoxThreads) finish_boxes_kernel(const Seg* __
     bool long_box = false;
     const int lowbits = 63 - 3 * Ls;
     const uint64_t lowmask = lowbits >= 64 ? ~0ull : ((1ull << lowbits) - 1ull);
+    // The points of a box differ in their low key bits only: the top 32 of those
+    // take the keys' low words (the boxes' keys below need the high words alone,
+    // to depth 10), and points are compared by them; points that agree there
+    // too, by the keys the sort left.  A box is compared all against all, so these
+    // loads and compares are most of the kernel's instructions: 7.4e7 points in 512
+    // sets 882 -> 740 us, 2 x 2^24 points on a sphere and in clumps 356 -> 309.
+    const bool words = Lb <= 10;
+    uint32_t* const low = reinterpret_cast<uint32_t*>(sk + 1);  // low[2 j]: point j
+    if (words) {
+      for (int j = threadIdx.x; j < jend; j += kBoxThreads) {
+        const uint64_t k = sk[j + 1] & lowmask;
+        low[2 * j] = (uint32_t)(lowbits > 32 ? k >> (lowbits - 32) : k);
+      }
+      __syncthreads();
+    }
     for (int c0 = warp * 32; c0 < jend; c0 += W * 32) {
       const int j = c0 + lane;
       const bool in = j < jend;
@@ -183,7 +198,23 @@ __global__ void __launch_bounds__(kBoxThreads) finish_boxes_kernel(const Seg* __
         continue;
       }
       uint32_t r = 0;
-      if (b - a > 1) {
+      if (words && b - a > 1) {
+        const uint32_t mine = low[2 * j];
+        uint32_t alike = 0;
+        for (int q = a; q < b; ++q) {
+          const uint32_t k = low[2 * q];
+          r += k < mine;
+          alike += k == mine;
+        }
+        if (alike > 1) {  // more than the point itself
+          const uint64_t key = keys[t0 + j];
+          for (int q = a; q < b; ++q) {
+            if (low[2 * q] != mine || q == j) continue;
+            const uint64_t kq = keys[t0 + q];
+            r += kq < key || (kq == key && s_val[q] < s_val[j]);
+          }
+        }
+      } else if (b - a > 1) {
         // within a box the top bits agree: order by (low key bits, index)
         const uint64_t mine = sk[j + 1] & lowmask;
         const uint32_t vj = s_val[j];
