@@ -37,39 +37,18 @@ namespace {
 
 __device__ __forceinline__ uint32_t bk_cells(int bl) { return 1u << (3 * bl); }
 
-// Bit i of v (v < 32) moved to bit 3i: the cell of level <= 5 from the top
-// bits of the three cell coordinates.
-__device__ __forceinline__ uint32_t spread5(uint32_t v) {
-  return (v & 1u) | ((v & 2u) << 2) | ((v & 4u) << 4) | ((v & 8u) << 6) | ((v & 16u) << 8);
+// Cell of one coordinate at level 21, saturated: the same as quantize21 for
+// coordinates in [0, 1], some cell for any other (a conversion takes negative
+// numbers and NaN to 0).
+__device__ __forceinline__ uint32_t quantize_sat(float x) {
+  return min((uint32_t)(x * 2097152.0f), 0x1fffffu);
 }
+__device__ __forceinline__ bool in_unit(float x) { return x >= 0.0f && x <= 1.0f; }
 
-// Bit i of a 21-bit value moved to bit 3i, by five shift-or-mask steps
-// (each halves the width of the bit groups still to be spread: 16, 8, 4, 2,
-// 1 bits, the masks keeping every group at its place).
-__device__ __forceinline__ uint64_t spread21(uint32_t x) {
-  uint64_t v = x & 0x1fffffu;
-  v = (v | (v << 32)) & 0x001f00000000ffffull;
-  v = (v | (v << 16)) & 0x001f0000ff0000ffull;
-  v = (v | (v << 8)) & 0x100f00f00f00f00full;
-  v = (v | (v << 4)) & 0x10c30c30c30c30c3ull;
-  v = (v | (v << 2)) & 0x1249249249249249ull;
-  return v;
-}
-// The same key as morton_key (same quantisation).
-__device__ __forceinline__ uint64_t spread_key(float x, float y, float z, bool* ok) {
-  uint32_t qx, qy, qz;
-  const bool a = quantize21(x, &qx), b = quantize21(y, &qy), c = quantize21(z, &qz);
-  *ok = a && b && c;
-  return spread21(qx) | (spread21(qy) << 1) | (spread21(qz) << 2);
-}
-
-// Cell of level bl (<= 5) of a point, and whether it lies in [0, 1]^3.
-__device__ __forceinline__ uint32_t cell_of(float x, float y, float z, int bl, bool* ok) {
-  uint32_t qx, qy, qz;
-  const bool a = quantize21(x, &qx), b = quantize21(y, &qy), c = quantize21(z, &qz);
-  *ok = a && b && c;
+// Cell of level bl (<= 10) of a point.
+__device__ __forceinline__ uint32_t cell_of(float x, float y, float z, int bl) {
   const int sh = 21 - bl;
-  return spread5(qx >> sh) | (spread5(qy >> sh) << 1) | (spread5(qz >> sh) << 2);
+  return interleave10(quantize_sat(x) >> sh, quantize_sat(y) >> sh, quantize_sat(z) >> sh);
 }
 
 // First level at which two items of one sub-cell of level bl1 differ (22:
@@ -246,19 +225,20 @@ __global__ void __launch_bounds__(kScThreads, 1) bucket_scatter_kernel(
     for (int u = 0; u < kScGroups; ++u) {
       const uint32_t g = g0 + u * kScThreads + threadIdx.x;
       if (g < ng) {
-        bool ok0, ok1, ok2, ok3;
-        atomicAdd(&s_at[cell_of(a[u].x, a[u].y, a[u].z, bl1, &ok0)], 1u);
-        atomicAdd(&s_at[cell_of(a[u].w, b[u].x, b[u].y, bl1, &ok1)], 1u);
-        atomicAdd(&s_at[cell_of(b[u].z, b[u].w, c[u].x, bl1, &ok2)], 1u);
-        atomicAdd(&s_at[cell_of(c[u].y, c[u].z, c[u].w, bl1, &ok3)], 1u);
-        bad |= !(ok0 && ok1 && ok2 && ok3);
+        atomicAdd(&s_at[cell_of(a[u].x, a[u].y, a[u].z, bl1)], 1u);
+        atomicAdd(&s_at[cell_of(a[u].w, b[u].x, b[u].y, bl1)], 1u);
+        atomicAdd(&s_at[cell_of(b[u].z, b[u].w, c[u].x, bl1)], 1u);
+        atomicAdd(&s_at[cell_of(c[u].y, c[u].z, c[u].w, bl1)], 1u);
+        bad |= !(in_unit(a[u].x) && in_unit(a[u].y) && in_unit(a[u].z) && in_unit(a[u].w) &&
+                 in_unit(b[u].x) && in_unit(b[u].y) && in_unit(b[u].z) && in_unit(b[u].w) &&
+                 in_unit(c[u].x) && in_unit(c[u].y) && in_unit(c[u].z) && in_unit(c[u].w));
       }
     }
   }
   for (uint32_t j = done + threadIdx.x; j < cnt; j += kScThreads) {
-    bool ok;
-    atomicAdd(&s_at[cell_of(xyz[3 * j], xyz[3 * j + 1], xyz[3 * j + 2], bl1, &ok)], 1u);
-    bad |= !ok;
+    const float x = xyz[3 * j], y = xyz[3 * j + 1], z = xyz[3 * j + 2];
+    atomicAdd(&s_at[cell_of(x, y, z, bl1)], 1u);
+    bad |= !(in_unit(x) && in_unit(y) && in_unit(z));
   }
   if (bad) set_error(st, FMM_ERR_DOMAIN);
   __syncthreads();
@@ -284,8 +264,7 @@ __global__ void __launch_bounds__(kScThreads, 1) bucket_scatter_kernel(
   // 3. the items, each at the next slot of its sub-cell's range
   uint64_t* const items = S.items;
   auto put = [&](float x, float y, float z, uint32_t j) {
-    bool ok;
-    const uint64_t key = spread_key(x, y, z, &ok);
+    const uint64_t key = interleave21(quantize_sat(x), quantize_sat(y), quantize_sat(z));
     const uint32_t sc = (uint32_t)(key >> sh);
     const uint32_t pos = atomicAdd(&s_at[sc], 1u);
     if (pos < (sc + 1u) * (uint32_t)kBkCap)  // (a sub-cell over its room keeps what fits)
