@@ -1064,6 +1064,13 @@ int run_build(fmm_ctx* c, std::vector<SetPlan>& sets, std::vector<JobPlan>& jobs
         std::max<uint32_t>(1, (uint32_t)(((uint64_t)sp.n + kBoxTile - 1) / kBoxTile));
     for (int l = 0; l <= sp.Lb; ++l) sp.cap[l] = level_cap(sp.n, l);
   }
+  uint64_t radix_boxes = 0;
+  int max_lb = 0;
+  for (auto& sp : sets) {
+    if (!sp.bucket) radix_boxes += sp.cap[sp.Lb];
+    max_lb = std::max(max_lb, sp.Lb);
+  }
+  const int citems = coarse_items(radix_boxes);
 
   // Zero-initialised words: the list sizes, then every set's tickets, box
   // counts and long-box flag side by side (one read-back copy for all of
@@ -1076,7 +1083,7 @@ int run_build(fmm_ctx* c, std::vector<SetPlan>& sets, std::vector<JobPlan>& jobs
   for (uint32_t i = 0; i < nsets; ++i) {
     zoff[i] = zero_bytes;
     zero_bytes += align_up(sizeof(uint64_t) * sets[i].dev.btiles) +
-                  align_up(sizeof(uint64_t) * coarse_tiles(sets[i].cap[sets[i].Lb]) * kLevels);
+                  align_up(sizeof(uint64_t) * coarse_tiles(sets[i].cap[sets[i].Lb], citems) * kLevels);
   }
   char* zero = arena_get<char>(c, std::max<size_t>(zero_bytes, 1), &err);
   if (err) return err;
@@ -1091,7 +1098,7 @@ int run_build(fmm_ctx* c, std::vector<SetPlan>& sets, std::vector<JobPlan>& jobs
     d.bstatus = reinterpret_cast<uint64_t*>(z);
     z += align_up(sizeof(uint64_t) * d.btiles);
     d.cstatus = reinterpret_cast<uint64_t*>(z);
-    z += align_up(sizeof(uint64_t) * coarse_tiles(sp.cap[sp.Lb]) * kLevels);
+    z += align_up(sizeof(uint64_t) * coarse_tiles(sp.cap[sp.Lb], citems) * kLevels);
     d.tickets = set_words + (size_t)i * kSetWords;
     d.nbox = d.tickets + 2;
     d.seg_long = d.nbox + kLevels;
@@ -1122,7 +1129,7 @@ int run_build(fmm_ctx* c, std::vector<SetPlan>& sets, std::vector<JobPlan>& jobs
     }
     if (sets[i].Lb >= 1 && !sets[i].bucket) {
       crs.push_back(Slot{i, m.crs_units, 0, 0});
-      m.crs_units += coarse_tiles(sets[i].cap[sets[i].Lb]);
+      m.crs_units += coarse_tiles(sets[i].cap[sets[i].Lb], citems);
     }
     if (sets[i].Lb >= 1 && sets[i].need_occ) {
       const uint32_t u = occupancy_units(sets[i].n);
@@ -1235,7 +1242,7 @@ int run_build(fmm_ctx* c, std::vector<SetPlan>& sets, std::vector<JobPlan>& jobs
       for (const Slot& o : occ)
         if (o.seg == set) {
           Launch L(c, "occupancy");
-          launch_occupancy(m.segs, m.occ_slots, (uint32_t)occ.size(), o.aux0, o.unit0, c->st, s);
+          launch_occupancy(m.segs, m.occ_slots, (uint32_t)occ.size(), o.aux0, o.unit0, max_lb, c->st, s);
         }
       return FMM_OK;
     };
@@ -1259,15 +1266,13 @@ int run_build(fmm_ctx* c, std::vector<SetPlan>& sets, std::vector<JobPlan>& jobs
     launch_sorted_xyz(m.segs, m.sx_slots, (uint32_t)sx.size(), sx_units, c->st, s);
   }
   if (m.crs_units) {
-    int max_lb = 0;
-    for (auto& sp : sets) max_lb = std::max(max_lb, sp.Lb);
     Launch L(c, "coarse_boxes");
-    launch_coarse_boxes(m.segs, m.crs_slots, (uint32_t)crs.size(), m.crs_units, max_lb, c->st,
+    launch_coarse_boxes(m.segs, m.crs_slots, (uint32_t)crs.size(), m.crs_units, max_lb, citems, c->st,
                         wait_ns, s);
   }
   if (m.occ_units && !early) {
     Launch L(c, "occupancy");
-    launch_occupancy(m.segs, m.occ_slots, (uint32_t)occ.size(), m.occ_units, 0, c->st, s);
+    launch_occupancy(m.segs, m.occ_slots, (uint32_t)occ.size(), m.occ_units, 0, max_lb, c->st, s);
   }
 
   // Reads the status word, the box counts and the list sizes back in one copy.
@@ -1838,7 +1843,7 @@ void workspace_parts(uint32_t N, uint32_t M, const fmm_params& p, uint64_t* byte
       if (bk > rx) total += bk - rx;
     }
     const uint64_t tiles = n / (kSortThreads * 4) + 1;  // the smallest tile
-    total += tiles * kRadixMax * 4 * 3 + (n / kBoxTile + 1) * 8 * (1 + kLevels);
+    total += tiles * kRadixMax * 4 * 3 + (n / (2 * kBoxThreads) + 1) * 8 * (1 + kLevels);
     total += tiles * sizeof(TileRec) * 8 + 8 * 256;  // tile records, 8 passes
     for (int l = 0; l <= L; ++l) total += align_up(21ull * level_cap(ns[k], l) + 8) + 1024;
   }

@@ -273,17 +273,22 @@ __global__ void __launch_bounds__(kBoxThreads) finish_boxes_kernel(const Seg* __
 // loops, unrolled, cover only the levels in use.
 // Four blocks an SM for trees up to level 8 (a few spilled registers): its
 // look-back waits hide better; deeper trees keep their registers.
-template <int NL>
-__global__ void __launch_bounds__(kBoxThreads, NL <= 8 ? 4 : 1) coarse_boxes_kernel(const Seg* __restrict__ segs,
+// ITEMS: boxes a thread.  A tile's chain of level scans, look-backs and stores is the
+// whole kernel for a few hundred thousand boxes: two boxes a thread then, eight
+// where the boxes alone fill the SMs (200003 clumped points, L = 6: 26 us with
+// eight, 16 with two; 10^6, L = 9: 33 and 27).
+template <int NL, int ITEMS>
+__global__ void __launch_bounds__(kBoxThreads, NL <= 8 ? 4 : (ITEMS == 2 && NL <= 12) ? 3 : 1) coarse_boxes_kernel(const Seg* __restrict__ segs,
                                                                    const Slot* __restrict__ slots,
                                                                    uint32_t nslots, DevStatus* st,
                                                                    uint64_t wait_ns) {
   constexpr int W = kBoxThreads / 32;
+  constexpr uint32_t kTile = kBoxThreads * ITEMS;
   __shared__ uint32_t s_tile, s_abort;
   __shared__ uint32_t s_wtot[W][kLevels];
   __shared__ uint32_t s_texcl[kLevels];
   __shared__ uint32_t s_ttot[kLevels];
-  __shared__ uint64_t s_key[kBoxTile + 1];  // s_key[j + 1] = level-Lb key of box t0 + j
+  __shared__ uint64_t s_key[kTile + 1];  // s_key[j + 1] = level-Lb key of box t0 + j
   grid_wait(segs, slots);
   const Seg& sg = segs[slots[find_slot(slots, nslots, blockIdx.x)].seg];
   const int Lb = sg.Lb;
@@ -299,21 +304,21 @@ __global__ void __launch_bounds__(kBoxThreads, NL <= 8 ? 4 : 1) coarse_boxes_ker
   __syncthreads();
   if (s_abort || Lb < 1) return;
   const uint32_t nb = nbox[Lb] < lv.cap[Lb] ? nbox[Lb] : lv.cap[Lb];
-  const uint32_t ntiles = nb == 0 ? 1u : (nb + kBoxTile - 1) / kBoxTile;
+  const uint32_t ntiles = nb == 0 ? 1u : (nb + kTile - 1) / kTile;
   const uint32_t tile = s_tile;
   if (tile >= ntiles) return;  // the grid is sized for the capacity
-  const int64_t t0 = (int64_t)tile * kBoxTile;
+  const int64_t t0 = (int64_t)tile * kTile;
   const uint64_t* kLb = lv.key[Lb];
   const int up = 63 - 3 * Lb;  // level-Lb key -> full-key position
-  for (int j = threadIdx.x; j < kBoxTile + 1; j += kBoxThreads) {
+  for (int j = threadIdx.x; j < kTile + 1; j += kBoxThreads) {
     const int64_t b = t0 - 1 + j;
     s_key[j] = (b >= 0 && b < (int64_t)nb) ? kLb[b] << up : 0ull;
   }
   __syncthreads();
-  uint32_t dd[kBoxItems];
+  uint32_t dd[ITEMS];
 #pragma unroll
-  for (int k = 0; k < kBoxItems; ++k) {
-    const int j = threadIdx.x * kBoxItems + k;
+  for (int k = 0; k < ITEMS; ++k) {
+    const int j = threadIdx.x * ITEMS + k;
     const int64_t b = t0 + j;
     dd[k] = b >= (int64_t)nb ? 0xffu : (b == 0 ? 0u : first_diff_level(s_key[j + 1], s_key[j]));
   }
@@ -324,7 +329,7 @@ __global__ void __launch_bounds__(kBoxThreads, NL <= 8 ? 4 : 1) coarse_boxes_ker
     if (l < Lb) {
       uint32_t c = 0;
 #pragma unroll
-      for (int k = 0; k < kBoxItems; ++k) c += (dd[k] <= (uint32_t)l);
+      for (int k = 0; k < ITEMS; ++k) c += (dd[k] <= (uint32_t)l);
       uint32_t x = c;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
@@ -371,8 +376,8 @@ __global__ void __launch_bounds__(kBoxThreads, NL <= 8 ? 4 : 1) coarse_boxes_ker
 #pragma unroll
   for (int l = 0; l < NL; ++l) run[l] = (l < Lb) ? s_texcl[l] + s_wtot[warp][l] + lex[l] : 0u;
 #pragma unroll
-  for (int k = 0; k < kBoxItems; ++k) {
-    const int j = threadIdx.x * kBoxItems + k;
+  for (int k = 0; k < ITEMS; ++k) {
+    const int j = threadIdx.x * ITEMS + k;
     const int64_t b = t0 + j;
     if (b >= (int64_t)nb) continue;
     const uint32_t dk = dd[k];
@@ -408,8 +413,10 @@ __global__ void __launch_bounds__(kBoxThreads, NL <= 8 ? 4 : 1) coarse_boxes_ker
   }
 }
 
-uint32_t coarse_tiles(uint32_t cap) {
-  const uint64_t t = ((uint64_t)cap + kBoxTile - 1) / kBoxTile;
+int coarse_items(uint64_t boxes) { return boxes <= (4u << 20) ? 2 : 8; }
+
+uint32_t coarse_tiles(uint32_t cap, int items) {
+  const uint64_t tile = (uint64_t)kBoxThreads * items, t = (cap + tile - 1) / tile;
   return t == 0 ? 1u : (uint32_t)t;
 }
 
@@ -426,17 +433,27 @@ void launch_finish_boxes(const Seg* segs, const Slot* slots, uint32_t nslots, ui
   launch_k(finish_boxes_kernel, units, kBoxThreads, kBoxSmem, s, segs, slots, nslots, st, wait_ns);
 }
 
+namespace {
+
+template <int ITEMS>
+void coarse_boxes_items(const Seg* segs, const Slot* slots, uint32_t nslots, uint32_t units,
+                        int max_lb, DevStatus* st, uint64_t wait_ns, cudaStream_t s) {
+  auto* const kernel = max_lb <= 8    ? coarse_boxes_kernel<8, ITEMS>
+                       : max_lb <= 12 ? coarse_boxes_kernel<12, ITEMS>
+                       : max_lb <= 16 ? coarse_boxes_kernel<16, ITEMS>
+                                      : coarse_boxes_kernel<kLevels, ITEMS>;
+  launch_k(kernel, units, kBoxThreads, 0, s, segs, slots, nslots, st, wait_ns);
+}
+
+}  // namespace
+
 void launch_coarse_boxes(const Seg* segs, const Slot* slots, uint32_t nslots, uint32_t units,
-                         int max_lb, DevStatus* st, uint64_t wait_ns, cudaStream_t s) {
+                         int max_lb, int items, DevStatus* st, uint64_t wait_ns, cudaStream_t s) {
   if (units == 0) return;
-  if (max_lb <= 8)
-    launch_k(coarse_boxes_kernel<8>, units, kBoxThreads, 0, s, segs, slots, nslots, st, wait_ns);
-  else if (max_lb <= 12)
-    launch_k(coarse_boxes_kernel<12>, units, kBoxThreads, 0, s, segs, slots, nslots, st, wait_ns);
-  else if (max_lb <= 16)
-    launch_k(coarse_boxes_kernel<16>, units, kBoxThreads, 0, s, segs, slots, nslots, st, wait_ns);
+  if (items == 2)
+    coarse_boxes_items<2>(segs, slots, nslots, units, max_lb, st, wait_ns, s);
   else
-    launch_k(coarse_boxes_kernel<kLevels>, units, kBoxThreads, 0, s, segs, slots, nslots, st, wait_ns);
+    coarse_boxes_items<8>(segs, slots, nslots, units, max_lb, st, wait_ns, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -444,18 +461,24 @@ void launch_coarse_boxes(const Seg* segs, const Slot* slots, uint32_t nslots, ui
 // as sources: bit o is set when the child in octant o (x + 2y + 4z) is
 // non-empty.  Lists use it to enumerate the children of a parent-level
 // neighbour without reading their keys.  A set owns a run of units (blocks)
-// in proportion to its size; each unit takes a strided share of every level.
+// in proportion to its size; a unit takes a strided share of one level, or in
+// builds that fill the SMs with units of every level in turn (a unit that walks
+// the levels waits three loads a level: 10^6 points, L = 9, 24 -> 16 us; 512 sets
+// have units enough, 78 us against 123).
 __global__ void __launch_bounds__(256) occupancy_kernel(const Seg* __restrict__ segs,
                                                         const Slot* __restrict__ slots,
                                                         uint32_t nslots, uint32_t unit_first,
+                                                        uint32_t launch_units,
                                                         const DevStatus* st) {
   grid_wait(segs, slots);
   if (failed(st)) return;
-  const uint32_t unit = blockIdx.x + unit_first;
+  const uint32_t unit = blockIdx.x % launch_units + unit_first;
+  const bool one_level = gridDim.x > launch_units;
+  const int l0 = (int)(blockIdx.x / launch_units);
   const uint32_t k = find_slot(slots, nslots, unit);
   const Seg& sg = segs[slots[k].seg];
   const uint32_t u = unit - slots[k].unit0, units = slots[k].aux0;
-  for (int l = 0; l < sg.Lb; ++l) {
+  for (int l = l0; l < (one_level ? min(l0 + 1, sg.Lb) : sg.Lb); ++l) {
     const uint32_t nb = sg.nbox[l] < sg.lv.cap[l] ? sg.nbox[l] : sg.lv.cap[l];
     const uint32_t* ch = sg.lv.child[l];
     const uint64_t* ck = sg.lv.key[l + 1];
@@ -471,9 +494,10 @@ __global__ void __launch_bounds__(256) occupancy_kernel(const Seg* __restrict__ 
 }
 
 void launch_occupancy(const Seg* segs, const Slot* slots, uint32_t nslots, uint32_t units,
-                      uint32_t unit_first, DevStatus* st, cudaStream_t s) {
-  if (units == 0) return;
-  launch_k(occupancy_kernel, units, 256, 0, s, segs, slots, nslots, unit_first, st);
+                      uint32_t unit_first, int max_lb, DevStatus* st, cudaStream_t s) {
+  if (units == 0 || max_lb == 0) return;
+  const uint32_t grid = units <= 304u ? units * (uint32_t)max_lb : units;
+  launch_k(occupancy_kernel, grid, 256, 0, s, segs, slots, nslots, unit_first, units, st);
 }
 
 uint32_t occupancy_units(uint32_t n) { return 1u + n / 16384u; }

@@ -548,7 +548,7 @@ void launch_finish_boxes(const Seg* segs, const Slot* slots, uint32_t nslots, ui
 // Levels 0..Lb-1, parents of level Lb, children of level Lb-1 (units =
 // coarse tiles by capacity).
 void launch_coarse_boxes(const Seg* segs, const Slot* slots, uint32_t nslots, uint32_t units,
-                         int max_lb, DevStatus* st, uint64_t wait_ns, cudaStream_t s);
+                         int max_lb, int items, DevStatus* st, uint64_t wait_ns, cudaStream_t s);
 // Child-occupancy bytes (sets flagged in `which`, grid y = set) and largest
 // occupancy per level.
 // Sorted points (xyz[perm[j]]) of the sets with `sorted` set; units: finishing tiles.
@@ -585,15 +585,17 @@ void launch_box_type(const fmm_tree& t, int l, int mode, const uint8_t* side, co
                      const uint8_t* border_up, uint8_t* border, uint8_t* on_next, uint8_t* type,
                      cudaStream_t s);
 // Child-occupancy bytes of the slots' sets (slot aux0 = the set's units):
-// the launch covers units [unit_first, unit_first + units).
+// the launch covers units [unit_first, unit_first + units) at levels below max_lb.
 void launch_occupancy(const Seg* segs, const Slot* slots, uint32_t nslots, uint32_t units,
-                      uint32_t unit_first, DevStatus* st, cudaStream_t s);
+                      uint32_t unit_first, int max_lb, DevStatus* st, cudaStream_t s);
 uint32_t occupancy_units(uint32_t n);
 // Cluster-size depth per set (units: sort tiles of the slots' sets); out[set]
 // = 1 + deepest level shared by sorted points i and i + s, capped at Ls.
 void launch_depth(const Seg* segs, const Slot* slots, uint32_t nslots, uint32_t units, uint32_t s,
                   uint32_t* out, DevStatus* st, cudaStream_t stream);
-uint32_t coarse_tiles(uint32_t cap);
+// Boxes a thread of a build whose radix sets have room for `boxes` finest boxes.
+int coarse_items(uint64_t boxes);
+uint32_t coarse_tiles(uint32_t cap, int items);
 
 // Exclusive scan of u32 counts in place (count entries at data[0..count)),
 // writes data[count] = total (low 32 bits) and total64 (if not null); flags
