@@ -7,7 +7,7 @@
 //   radix passes (per-tile digit histograms -> one prefix sum -> scatter; the
 //   first pass forms the Morton keys from the coordinates) -> finishing sort
 //   inside boxes + finest boxes -> coarser boxes -> child occupancy;
-// then per level l = 2..L two launches for the lists.
+// then per level l = 2..L one or two launches for the lists.
 // The host synchronises once at the end, and also: in cluster-size mode after
 // the sort (to learn each set's depth) and after the full-key sort of the sets
 // that need one; when the list capacity bound is too large, after the boxes.
@@ -1180,6 +1180,7 @@ int run_build(fmm_ctx* c, std::vector<SetPlan>& sets, std::vector<JobPlan>& jobs
 
   // List arrays (per level, shared by the jobs) and per-job row starts.
   std::vector<uint32_t> chunks(kLevels, 0);
+  std::vector<uint64_t> lparents(kLevels, 0);
   char* list_zero = nullptr;
   size_t list_zero_bytes = 0;
   auto plan_lists = [&]() -> int {
@@ -1201,14 +1202,23 @@ int run_build(fmm_ctx* c, std::vector<SetPlan>& sets, std::vector<JobPlan>& jobs
       }
       if (rows >= (1ull << 32) || room[l] >= (1ull << 32)) return FMM_ERR_CAPACITY;
       chunks[l] = list_chunks(parents, njobs);
+      lparents[l] = parents;
       zo[l] = list_zero_bytes;
       list_zero_bytes += align_up(sizeof(uint32_t));
+      if (list_small(njobs, parents))
+        list_zero_bytes += 2 * align_up(sizeof(uint64_t) * list_small_tiles(parents));
     }
     list_zero = arena_get<char>(c, std::max<size_t>(list_zero_bytes, 1), &err);
     if (err) return err;
     for (int l = 2; l <= Lmax; ++l) {
       ListLevel& LV = lvls[l];
       LV.ticket = reinterpret_cast<uint32_t*>(list_zero + zo[l]);
+      if (list_small(njobs, lparents[l])) {
+        char* z = list_zero + zo[l] + align_up(sizeof(uint32_t));
+        LV.status2 = reinterpret_cast<uint64_t*>(z);
+        LV.status4 = reinterpret_cast<uint64_t*>(
+            z + align_up(sizeof(uint64_t) * list_small_tiles(lparents[l])));
+      }
       LV.nnz = nnz_words + (size_t)l * njobs * 2;
       LV.off2 = arena_get<uint32_t>(c, 4ull * chunks[l], &err);
       LV.off4 = arena_get<uint32_t>(c, 4ull * chunks[l], &err);
@@ -1315,6 +1325,11 @@ int run_build(fmm_ctx* c, std::vector<SetPlan>& sets, std::vector<JobPlan>& jobs
   }
   for (int l = 2; l <= Lmax; ++l) {
     const LevelJob one = level_job(jobs[0].dev, sets[jobs[0].src].dev, sets[jobs[0].recv].dev, l, lvls[l - 1]);
+    if (list_small(njobs, lparents[l])) {
+      Launch Lk(c, "list_small");
+      launch_list_small(l, lvls[l], lvls[l - 1], one, lparents[l], c->st, wait_ns, s);
+      continue;
+    }
     {
       Launch Lk(c, "list_count");
       launch_list_count(m.segs, m.jobs, njobs, l, lvls[l], lvls[l - 1], one, chunks[l], c->st, s);

@@ -419,7 +419,9 @@ struct ListLevel {
   uint32_t* off4;
   uint64_t* bbase;   // [list_blocks()][2] first E2 / E4 entries of the count blocks
   uint64_t* jbase;   // [njobs][2] ... and of the jobs
-  uint32_t* ticket;  // count blocks done (zeroed)
+  uint64_t* status2; // [list_small_tiles] look-back words of the E2 / E4 entries (zeroed; small
+  uint64_t* status4; // levels, else null)
+  uint32_t* ticket;  // count blocks done, or small-level blocks taken (zeroed)
   uint64_t* nnz;     // [njobs][2] E2 / E4 entries of each job (zeroed)
 };
 
@@ -615,6 +617,12 @@ uint32_t scan_tiles(uint32_t cap);
 LevelJob level_job(const Job& J, const Seg& src, const Seg& recv, int l, const ListLevel& up);
 uint32_t list_chunks(uint64_t cap, uint32_t njobs);
 uint32_t list_blocks();
+// Whether a level of at most `parents` parents takes launch_list_small instead of
+// the count and the fill, and its blocks.
+bool list_small(uint32_t njobs, uint64_t parents);
+uint32_t list_small_tiles(uint64_t parents);
+void launch_list_small(int l, const ListLevel& lv, const ListLevel& up, const LevelJob& one,
+                       uint64_t parents, DevStatus* st, uint64_t wait_ns, cudaStream_t s);
 void launch_list_plan(const Seg* segs, const Job* jobs, uint32_t njobs, int Lmax,
                       const ListLevel* lvls, DevStatus* st, cudaStream_t s);
 void launch_list_count(const Seg* segs, const Job* jobs, uint32_t njobs, int l,

@@ -17,7 +17,7 @@
 // and walking Q in ascending rank, children in ascending octant, yields
 // ascending ranks.
 //
-// Two launches a level.  The count kernel finds every parent's E2 and E4
+// Two launches a level (one for small levels of one job).  The count kernel finds every parent's E2 and E4
 // entries and their prefix sums (of its receiver children together); the fill kernel
 // writes rows and entries, one warp a parent, no warp waiting for another.
 // Both walk the parents in chunks of four that never cross a job (a job's last
@@ -127,6 +127,9 @@ __device__ __forceinline__ uint32_t job_chunks(const Job& J, const Seg* segs, in
 // Chunks of a level of at most `cap` parents in all, at most.
 uint32_t list_chunks(uint64_t cap, uint32_t njobs) { return (uint32_t)(cap / kChunk) + njobs; }
 uint32_t list_blocks() { return kCountGrid; }
+uint32_t list_small_tiles(uint64_t parents) {
+  return (uint32_t)std::max<uint64_t>((parents + kFillWarps - 1) / kFillWarps, 1u);
+}
 
 // Per level (one block each): the chunks before each job.
 __global__ void __launch_bounds__(1024) list_plan_kernel(const Seg* __restrict__ segs,
@@ -537,13 +540,24 @@ __device__ __forceinline__ void each_sibling(uint32_t nsib, const F& f) {
   }
 }
 
-// One parent: its siblings' rows and entries.  kWide: more than four siblings.
-template <bool kCodes, bool kWide>
+// The job's lists of the level: rows, entries and offset codes.
+struct FillOut {
+  uint32_t *out2, *out4, *idx2, *idx4;
+  uint8_t* code2;
+};
+// A parent's first entries in the job's lists; no place: a wait gave up.
+struct Place {
+  uint64_t e2, e4;
+  bool ok;
+};
+
+// One parent: its siblings' rows and entries.  kWide: more than four siblings.  c0:
+// its first receiver child; place(E2 entries, E4 entries) gives its place.
+template <bool kCodes, bool kWide, class PlaceFn>
 __device__ __forceinline__ void fill_parent(FillWarp& F, uint2 mk, uint32_t sel, uint32_t nsib,
                                             uint32_t occ, uint32_t code, uint32_t rank,
-                                            uint32_t present, uint32_t* out2, uint32_t* out4,
-                                            uint32_t at2, uint32_t at4, uint32_t* e2, uint32_t* e4,
-                                            uint8_t* codes) {
+                                            uint32_t present, uint32_t c0, const FillOut& o_,
+                                            const PlaceFn& place) {
   const int lane = threadIdx.x & 31;
   // child masks of the siblings, in their order; none for absent ones
   uint32_t m0 = __byte_perm(mk.x, mk.y, sel), m1 = 0;
@@ -570,10 +584,16 @@ __device__ __forceinline__ void fill_parent(FillWarp& F, uint2 mk, uint32_t sel,
     tw = __shfl_sync(0xffffffffu, xh, 31);
     f1 = tw * 0x01010100u + byte_sum(tl) * 0x01010101u;
   }
+  const uint32_t n2 = byte_sum(tl) + (kWide ? byte_sum(tw) : 0u);
+  const Place at = place(n2, nsib * total - n2);
+  if (!at.ok) return;
+  uint32_t* const e2 = o_.idx2 + at.e2;
+  uint32_t* const e4 = o_.idx4 + at.e4;
+  uint8_t* const codes = kCodes ? o_.code2 + at.e2 : nullptr;
   if ((uint32_t)lane < nsib) {
     const uint32_t f = ((kWide && lane >= 4 ? f1 : f0) >> (8 * (lane & 3))) & 0xffu;
-    out2[lane] = at2 + f;
-    out4[lane] = at4 + lane * total - f;
+    o_.out2[c0 + lane] = (uint32_t)at.e2 + f;
+    o_.out4[c0 + lane] = (uint32_t)at.e4 + lane * total - f;
   }
   uint32_t lo = xl - lo0 + f0, hi = xh - hi0 + f1;
   uint32_t e = (xc - cn) & 0xffffu, ne = (xc - cn) >> 16;
@@ -763,25 +783,147 @@ __global__ void __launch_bounds__(kListThreads, 4) list_fill_kernel(
       if (k < k0) continue;
       const uint32_t present = __shfl_sync(0xffffffffu, octs, 8 * k);
       const uint32_t c0 = __shfl_sync(0xffffffffu, head, 8 + k);
-      const uint64_t at2 = g2 + __shfl_sync(0xffffffffu, head, 16 + k);
-      const uint64_t at4 = g4 + __shfl_sync(0xffffffffu, head, 24 + k);
+      const Place at{g2 + __shfl_sync(0xffffffffu, head, 16 + k),
+                     g4 + __shfl_sync(0xffffffffu, head, 24 + k), true};
+      const auto place = [&](uint32_t, uint32_t) { return at; };
       const uint32_t nsib = __popc(present);
       const uint64_t slot = W.slot;
-      uint32_t* const e2 = LV.idx2 + 27ull * slot + at2;
-      uint32_t* const e4 = LV.idx4 + 189ull * slot + at4;
-      uint8_t* const codes = kCodes ? LV.code2 + 27ull * slot + at2 : nullptr;
+      const FillOut out{W.out2, W.out4, LV.idx2 + 27ull * slot, LV.idx4 + 189ull * slot,
+                        kCodes ? LV.code2 + 27ull * slot : nullptr};
       const uint2 mk = sm.mask[co >> 8];
       const uint32_t sel = sm.sel[present];
       if (nsib > 4)
-        fill_parent<kCodes, true>(F, mk, sel, nsib, co & 0xffu, co >> 8, rank, present,
-                                  W.out2 + c0, W.out4 + c0, (uint32_t)at2, (uint32_t)at4, e2, e4,
-                                  codes);
+        fill_parent<kCodes, true>(F, mk, sel, nsib, co & 0xffu, co >> 8, rank, present, c0, out, place);
       else if (nsib > 0)
-        fill_parent<kCodes, false>(F, mk, sel, nsib, co & 0xffu, co >> 8, rank, present,
-                                   W.out2 + c0, W.out4 + c0, (uint32_t)at2, (uint32_t)at4, e2, e4,
-                                   codes);
+        fill_parent<kCodes, false>(F, mk, sel, nsib, co & 0xffu, co >> 8, rank, present, c0, out, place);
     }
   }
+}
+
+// Levels of one job whose parents fit one a warp of a resident grid: counts, prefix
+// sums and entries in one launch.  A block takes eight parents (in order, by
+// ticket); their counts go up a decoupled look-back over the blocks, E2 by warp 0
+// and E4 by warp 1, while the parents' candidates wait in registers.  Levels 2..4
+// of 16384 points: 32 us in three launches, 58 in the six of count and fill; above
+// a resident grid's parents the look-backs and barriers cost more than a second
+// launch (512 sets in one launch a level: 5.96 ms, 3.47 in two).
+template <bool kCodes>
+__global__ void __launch_bounds__(kListThreads, 4) list_small_kernel(
+    int l, const __grid_constant__ ListLevel LV, const __grid_constant__ ListLevel up,
+    const __grid_constant__ LevelJob W, DevStatus* st, uint64_t wait_ns) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  FillSmem& sm = *reinterpret_cast<FillSmem*>(smem_raw);
+  __shared__ uint32_t s_tile, s_stop, s_n[2][kFillWarps];
+  __shared__ uint64_t s_base[2];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (tid < kNbor) sm.mask[tid] = code_masks(tid);
+  if (tid < 256) {
+    uint32_t sel = 0, n = 0;
+    for (uint32_t rho = 0; rho < 8; ++rho)
+      if ((tid >> rho) & 1) sel |= rho << (4 * n++);
+    sm.sel[tid] = sel;
+  }
+  grid_wait();
+  const uint32_t np = W.rnbox[l - 1];
+  if (tid == 0) {
+    s_stop = failed(st) ? 1u : 0u;
+    s_tile = atomicAdd(LV.ticket, 1u);
+  }
+  __syncthreads();
+  const uint32_t tile = s_tile, tiles = max((np + kFillWarps - 1) / kFillWarps, 1u);
+  if (s_stop || tile >= tiles) return;
+  const uint32_t p = tile * kFillWarps + warp;
+
+  // The parent's row, children, neighbours (one a lane) and receiver octants.
+  uint32_t co = 13u << 8, rank = 0, present = 0, c0 = 0;
+  if (p < np) {
+    const uint32_t head = lane < 2   ? (l == 2 ? 0u : W.off_up[p + lane])
+                          : lane < 4 ? W.rchild[p + lane - 2]
+                                     : 0u;
+    const uint32_t first = __shfl_sync(0xffffffffu, head, 0);
+    const uint32_t m = l == 2 ? min(W.snbox[1], 8u)
+                              : min(__shfl_sync(0xffffffffu, head, 1) - first, (uint32_t)kNbor);
+    c0 = __shfl_sync(0xffffffffu, head, 2);
+    const uint32_t nch = min(__shfl_sync(0xffffffffu, head, 3) - c0, 8u);
+    const uint32_t oct = (uint32_t)lane < nch ? 1u << (uint32_t)(W.rkey[c0 + lane] & 7u) : 0u;
+    if ((uint32_t)lane < m) {
+      uint32_t q = lane;
+      if (l == 2) {
+        co = level1_code((uint32_t)W.skey1[lane], (uint32_t)W.rkey1[p]) << 8;
+      } else {
+        q = W.idx_up[first + lane];
+        co = (uint32_t)W.code_up[first + lane] << 8;
+      }
+      co |= W.socc[q];
+      rank = W.schild[q];
+    }
+    present = __reduce_or_sync(0xffffffffu, oct);
+  }
+  // The block's counts and their place.  Every warp comes here once, from its own
+  // call of fill_parent or, without a parent, from below: named barriers.
+  const auto place = [&](uint32_t n2, uint32_t n4) {
+    if (lane == 0) {
+      s_n[0][warp] = n2;
+      s_n[1][warp] = n4;
+    }
+    __syncwarp();
+    asm volatile("barrier.sync 1, %0;" ::"n"(kListThreads) : "memory");
+    if (warp < 2) {
+      uint64_t* const chain = warp ? LV.status4 : LV.status2;
+      const uint32_t v = lane < kFillWarps ? s_n[warp][lane] : 0u;
+      const uint32_t x = warp_incl(v), tot = __shfl_sync(0xffffffffu, x, 31);
+      uint64_t prev = 0;
+      if (lane == 0) st_relaxed(chain + tile, (tile == 0 ? kFlagIncl : kFlagAgg) | tot);
+      if (tile > 0) {
+        prev = lookback_warp(chain, tile, 1, st, wait_ns);
+        if (lane == 0) st_relaxed(chain + tile, kFlagIncl | (prev + tot));
+      }
+      if (lane < kFillWarps) s_n[warp][lane] = x - v;
+      if (lane == 0) {
+        s_base[warp] = prev;
+        if (tile > 0 && ld_relaxed_u32(&st->abort)) s_stop = 1;
+        if (tile + 1 == tiles) {  // the last block closes the rows
+          const uint64_t n = prev + tot;
+          (warp ? W.out4 : W.out2)[W.rnbox[l]] = (uint32_t)n;
+          LV.nnz[warp] = n;
+          if (n >> 32) set_error(st, FMM_ERR_CAPACITY);
+        }
+      }
+      __syncwarp();
+    }
+    asm volatile("barrier.sync 1, %0;" ::"n"(kListThreads) : "memory");
+    return Place{s_base[0] + s_n[0][warp], s_base[1] + s_n[1][warp], s_stop == 0};
+  };
+  const uint32_t nsib = __popc(present);
+  const FillOut out{W.out2, W.out4, LV.idx2 + 27ull * W.slot, LV.idx4 + 189ull * W.slot,
+                    kCodes ? LV.code2 + 27ull * W.slot : nullptr};
+  const uint2 mk = sm.mask[co >> 8];
+  const uint32_t sel = sm.sel[present];
+  if (nsib > 4)
+    fill_parent<kCodes, true>(sm.w[warp], mk, sel, nsib, co & 0xffu, co >> 8, rank, present, c0, out, place);
+  else if (nsib > 0)
+    fill_parent<kCodes, false>(sm.w[warp], mk, sel, nsib, co & 0xffu, co >> 8, rank, present, c0, out, place);
+  else
+    place(0, 0);
+}
+
+bool list_small(uint32_t njobs, uint64_t parents) {
+  return njobs == 1 && parents <= (uint64_t)kFillGrid * kFillWarps;
+}
+
+void launch_list_small(int l, const ListLevel& lv, const ListLevel& up, const LevelJob& one,
+                       uint64_t parents, DevStatus* st, uint64_t wait_ns, cudaStream_t s) {
+  static const bool attr = [] {
+    cudaFuncSetAttribute(list_small_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)sizeof(FillSmem));
+    cudaFuncSetAttribute(list_small_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)sizeof(FillSmem));
+    return true;
+  }();
+  (void)attr;
+  const uint32_t grid = list_small_tiles(parents);
+  launch_k(lv.code2 ? list_small_kernel<true> : list_small_kernel<false>, grid, kListThreads,
+           sizeof(FillSmem), s, l, lv, up, one, st, wait_ns);
 }
 
 void launch_list_count(const Seg* segs, const Job* jobs, uint32_t njobs, int l,

@@ -44,6 +44,13 @@ def test_box_occupancies(ctx, orc, L, share):
         compare_full(ctx.build(_dev(a), _dev(b), L=L).numpy(), orc.build_tree(a, b, L=L), L)
 
 
+@pytest.mark.parametrize("m", [1, 4863, 4864, 4865, 4872])
+def test_one_launch_or_two(ctx, orc, m):
+    """Around the parents that one launch a level takes (608 blocks of eight)."""
+    src, recv = workloads.uniform(6000, 3), workloads.uniform(m, m)
+    compare_full(ctx.build(_dev(src), _dev(recv), L=7).numpy(), orc.build_tree(src, recv, L=7), 7)
+
+
 def test_jobs_without_points(ctx, orc):
     none = np.zeros((0, 3), np.float32)
     pairs = [(_subset(4, 0.4, k), _subset(4, 0.6, 50 + k)) for k in range(7)]
