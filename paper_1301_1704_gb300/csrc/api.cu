@@ -560,7 +560,7 @@ char* upload(fmm_ctx* c, const Upload& up, int* err, void* z0 = nullptr, size_t 
   }
   char* h = static_cast<char*>(c->up_buf) + c->up_cursor;
   std::memcpy(h, up.bytes.data(), need);
-  // the device reads the pinned staging buffer directly (see copy_words_kernel)
+  // the device reads the pinned staging buffer directly (copy_zero_kernel)
   void* hd = nullptr;
   if (cudaHostGetDevicePointer(&hd, h, 0) != cudaSuccess) {
     cudaGetLastError();

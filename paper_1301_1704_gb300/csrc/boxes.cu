@@ -265,29 +265,79 @@ __global__ void __launch_bounds__(kBoxThreads) finish_boxes_kernel(const Seg* __
   }
 }
 
+// Box starts of a box whose key first differs from the one before it at level dk: one
+// at every level from dk on, counted in the halves of a level pair's word.
+__device__ __forceinline__ uint32_t opens(uint32_t dk, int pair) {
+  return dk <= 2u * pair ? 0x10001u : (dk == 2u * pair + 1u ? 0x10000u : 0u);
+}
+
+// A thread's ITEMS consecutive words (aligned like ITEMS words), `have` of them there.
+template <int ITEMS>
+__device__ __forceinline__ void load_items(uint32_t (&v)[ITEMS], const uint32_t* p, bool whole,
+                                           int64_t have) {
+  if (whole) {
+    if constexpr (ITEMS == 2) {
+      const uint2 a = *reinterpret_cast<const uint2*>(p);
+      v[0] = a.x, v[1] = a.y;
+    } else {
+#pragma unroll
+      for (int k = 0; k < ITEMS; k += 4) {
+        const uint4 a = *reinterpret_cast<const uint4*>(p + k);
+        v[k] = a.x, v[k + 1] = a.y, v[k + 2] = a.z, v[k + 3] = a.w;
+      }
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < ITEMS; ++k) v[k] = k < have ? p[k] : 0u;
+  }
+}
+
+template <int ITEMS>
+__device__ __forceinline__ void store_items(uint32_t* p, const uint32_t (&v)[ITEMS], bool whole,
+                                            int64_t have) {
+  if (whole) {
+    if constexpr (ITEMS == 2) {
+      *reinterpret_cast<uint2*>(p) = make_uint2(v[0], v[1]);
+    } else {
+#pragma unroll
+      for (int k = 0; k < ITEMS; k += 4)
+        *reinterpret_cast<uint4*>(p + k) = make_uint4(v[k], v[k + 1], v[k + 2], v[k + 3]);
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < ITEMS; ++k)
+      if (k < have) p[k] = v[k];
+  }
+}
+
 // Levels 0..Lb-1 (and the parents of the level-Lb boxes) from the level-Lb
 // boxes: box b opens a level-l box exactly when its key differs from box
 // b-1's in the level-l prefix.  A multi-level prefix sum over the boxes (one
 // decoupled look-back chain per level) gives each start its rank.
 // NL: a bound on the sets' box depths (Lb <= NL), so that the per-level
 // loops, unrolled, cover only the levels in use.
-// Four blocks an SM for trees up to level 8 (a few spilled registers): its
-// look-back waits hide better; deeper trees keep their registers.
+// Bound by latency (the look-backs, and stores that follow loads), so: the level-Lb
+// bookmarks are loaded before the scans, eight a thread in two vectors; starts are
+// counted two levels to a word, which halves the shuffles and lets two blocks of up
+// to twelve levels share an SM (one did before); a thread's parents leave as vectors.
+// 2 x 2^24 points on a sphere and in clumps, L = 9: 242 -> 133 us; 512 sets of
+// 7.4e7 points: 540 -> 277 us.
 // ITEMS: boxes a thread.  A tile's chain of level scans, look-backs and stores is the
 // whole kernel for a few hundred thousand boxes: two boxes a thread then, eight
 // where the boxes alone fill the SMs (200003 clumped points, L = 6: 26 us with
 // eight, 16 with two; 10^6, L = 9: 33 and 27).
 template <int NL, int ITEMS>
-__global__ void __launch_bounds__(kBoxThreads, NL <= 8 ? 4 : (ITEMS == 2 && NL <= 12) ? 3 : 1) coarse_boxes_kernel(const Seg* __restrict__ segs,
+__global__ void __launch_bounds__(kBoxThreads, NL <= 8 ? (ITEMS == 2 ? 4 : 3) : NL <= 12 ? (ITEMS == 2 ? 3 : 2) : 1) coarse_boxes_kernel(const Seg* __restrict__ segs,
                                                                    const Slot* __restrict__ slots,
                                                                    uint32_t nslots, DevStatus* st,
                                                                    uint64_t wait_ns) {
   constexpr int W = kBoxThreads / 32;
   constexpr uint32_t kTile = kBoxThreads * ITEMS;
   __shared__ uint32_t s_tile, s_abort;
-  __shared__ uint32_t s_wtot[W][kLevels];
-  __shared__ uint32_t s_texcl[kLevels];
-  __shared__ uint32_t s_ttot[kLevels];
+  constexpr int NP = (NL + 1) / 2;  // level pairs: a tile's counts fit 16 bits
+  __shared__ uint32_t s_wtot[W][NP];     // a warp's box starts, two levels to a word
+  __shared__ uint32_t s_wex[W][kLevels]; // rank of a warp's first start
+  __shared__ uint32_t s_ttot[kLevels];   // rank after the tile's last start
   __shared__ uint64_t s_key[kTile + 1];  // s_key[j + 1] = level-Lb key of box t0 + j
   grid_wait(segs, slots);
   const Seg& sg = segs[slots[find_slot(slots, nslots, blockIdx.x)].seg];
@@ -322,43 +372,49 @@ __global__ void __launch_bounds__(kBoxThreads, NL <= 8 ? 4 : (ITEMS == 2 && NL <
     const int64_t b = t0 + j;
     dd[k] = b >= (int64_t)nb ? 0xffu : (b == 0 ? 0u : first_diff_level(s_key[j + 1], s_key[j]));
   }
-  uint32_t lex[NL];
+  // Level-Lb bookmarks of the thread's boxes, on their way during the scans.
+  uint32_t off[ITEMS];
+  const uint32_t* kOff = lv.off[Lb] + t0 + threadIdx.x * ITEMS;  // 4 * ITEMS-byte aligned
+  const bool whole = t0 + (int64_t)(threadIdx.x + 1) * ITEMS <= (int64_t)nb;
+  load_items<ITEMS>(off, kOff, whole, (int64_t)nb - t0 - threadIdx.x * ITEMS);
+  uint32_t run[NP];
 #pragma unroll
-  for (int l = 0; l < NL; ++l) {
-    lex[l] = 0;
-    if (l < Lb) {
+  for (int p = 0; p < NP; ++p) {
+    run[p] = 0;
+    if (2 * p < Lb) {
       uint32_t c = 0;
 #pragma unroll
-      for (int k = 0; k < ITEMS; ++k) c += (dd[k] <= (uint32_t)l);
+      for (int k = 0; k < ITEMS; ++k) c += opens(dd[k], p);
       uint32_t x = c;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
         const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
         if (lane >= o) x += y;
       }
-      lex[l] = x - c;
-      if (lane == 31) s_wtot[warp][l] = x;
+      run[p] = x - c;
+      if (lane == 31) s_wtot[warp][p] = x;
     }
   }
   __syncthreads();
   for (int l = warp; l < Lb; l += W) {
-    if (lane == 0) {
-      uint32_t run = 0;
-      for (int w = 0; w < W; ++w) {
-        const uint32_t c = s_wtot[w][l];
-        s_wtot[w][l] = run;
-        run += c;
-      }
-      s_ttot[l] = run;
-      st_relaxed(status + (uint64_t)tile * kLevels + l, (tile == 0 ? kFlagIncl : kFlagAgg) | run);
+    const uint32_t c = lane < W ? (s_wtot[lane][l >> 1] >> (16 * (l & 1))) & 0xffffu : 0u;
+    uint32_t x = c;
+#pragma unroll
+    for (int o = 1; o < W; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
     }
+    const uint32_t total = __shfl_sync(0xffffffffu, x, W - 1);
+    if (lane == 0)
+      st_relaxed(status + (uint64_t)tile * kLevels + l, (tile == 0 ? kFlagIncl : kFlagAgg) | total);
     uint64_t prev = 0;
     if (tile > 0) {
       prev = lookback_warp(status + l, tile, kLevels, st, wait_ns);
-      if (lane == 0)
-        st_relaxed(status + (uint64_t)tile * kLevels + l, kFlagIncl | (prev + s_ttot[l]));
+      if (lane == 0) st_relaxed(status + (uint64_t)tile * kLevels + l, kFlagIncl | (prev + total));
     }
-    if (lane == 0) s_texcl[l] = (uint32_t)prev;
+    prev = __shfl_sync(0xffffffffu, (uint32_t)prev, 0);
+    if (lane < W) s_wex[lane][l] = (uint32_t)prev + x - c;
+    if (lane == 0) s_ttot[l] = (uint32_t)prev + total;
   }
   __syncthreads();
   if (threadIdx.x == 0 && tile > 0 && ld_relaxed_u32(&st->abort)) s_abort = 1;
@@ -366,51 +422,53 @@ __global__ void __launch_bounds__(kBoxThreads, NL <= 8 ? 4 : (ITEMS == 2 && NL <
   if (s_abort) return;  // a wait gave up: ranks may be wrong, write nothing
   if (tile == ntiles - 1 && threadIdx.x == 0) {
     for (int l = 0; l < Lb; ++l) {
-      const uint32_t c = s_texcl[l] + s_ttot[l];
+      const uint32_t c = s_ttot[l];
       nbox[l] = c;
       if (c <= lv.cap[l]) lv.off[l][c] = n;
-      if (c <= lv.cap[l]) lv.child[l][c] = l + 1 < Lb ? s_texcl[l + 1] + s_ttot[l + 1] : nb;
+      if (c <= lv.cap[l]) lv.child[l][c] = l + 1 < Lb ? s_ttot[l + 1] : nb;
     }
   }
-  uint32_t run[NL];
+  // the next level-(Lb-1) box's rank: a level-Lb box's parent is the one before
+  uint32_t last = s_wex[warp][Lb - 1];
 #pragma unroll
-  for (int l = 0; l < NL; ++l) run[l] = (l < Lb) ? s_texcl[l] + s_wtot[warp][l] + lex[l] : 0u;
+  for (int p = 0; p < NP; ++p)
+    if (p == (Lb - 1) >> 1) last += (run[p] >> (16 * ((Lb - 1) & 1))) & 0xffffu;
+  uint32_t par[ITEMS];
 #pragma unroll
   for (int k = 0; k < ITEMS; ++k) {
     const int j = threadIdx.x * ITEMS + k;
-    const int64_t b = t0 + j;
-    if (b >= (int64_t)nb) continue;
     const uint32_t dk = dd[k];
-    const uint64_t key = s_key[j + 1];
-    // parent of the level-Lb box: the level-(Lb-1) box holding it
-    if (Lb >= 1) {
-      uint32_t pr = 0;
-#pragma unroll
-      for (int l = 0; l < NL; ++l)
-        if (l == Lb - 1) pr = dk <= (uint32_t)l ? run[l] : run[l] - 1u;
-      lv.parent[Lb][b] = pr;
-      if (dk <= (uint32_t)(Lb - 1) && pr < lv.cap[Lb - 1]) lv.child[Lb - 1][pr] = (uint32_t)b;
-    }
     if (dk < (uint32_t)Lb) {
-      const uint32_t off = lv.off[Lb][b];
+      const uint64_t key = s_key[j + 1];
+      if (last < lv.cap[Lb - 1]) lv.child[Lb - 1][last] = (uint32_t)t0 + j;
+      ++last;
+      uint32_t up_rk = 0;  // rank of the level-(l-1) box open at this box or before it
 #pragma unroll
       for (int l = 0; l < NL; ++l) {
-        if (l < Lb && (uint32_t)l >= dk && run[l] < lv.cap[l]) {
-          const uint32_t rk = run[l];
-          lv.key[l][rk] = l == 0 ? 0ull : key >> (63 - 3 * l);
-          lv.off[l][rk] = off;
-          if (l >= 1) {
-            const bool up_starts = dk <= (uint32_t)(l - 1);
-            lv.parent[l][rk] = up_starts ? run[l - 1] : run[l - 1] - 1u;
-            if (up_starts && run[l - 1] < lv.cap[l - 1]) lv.child[l - 1][run[l - 1]] = rk;
+        if (l < Lb && l + 1 >= (int)dk) {
+          const uint32_t rk = s_wex[warp][l] + ((run[l / 2] >> (16 * (l & 1))) & 0xffffu);
+          if ((uint32_t)l >= dk) {
+            if (rk < lv.cap[l]) {
+              lv.key[l][rk] = l == 0 ? 0ull : key >> (63 - 3 * l);
+              lv.off[l][rk] = off[k];
+              if (l >= 1) {
+                lv.parent[l][rk] = up_rk;
+                if ((uint32_t)l > dk && up_rk < lv.cap[l - 1]) lv.child[l - 1][up_rk] = rk;
+              }
+            }
+            up_rk = rk;
+          } else {
+            up_rk = rk - 1u;  // l = dk - 1: the last box of the level so far
           }
         }
       }
     }
+    par[k] = last - 1u;
 #pragma unroll
-    for (int l = 0; l < NL; ++l)
-      if (l < Lb && (uint32_t)l >= dk) ++run[l];
+    for (int p = 0; p < NP; ++p) run[p] += opens(dk, p);
   }
+  store_items<ITEMS>(lv.parent[Lb] + t0 + threadIdx.x * ITEMS, par, whole,
+                     (int64_t)nb - t0 - threadIdx.x * ITEMS);
 }
 
 int coarse_items(uint64_t boxes) { return boxes <= (4u << 20) ? 2 : 8; }
