@@ -9,7 +9,7 @@
 //   inside boxes + finest boxes -> coarser boxes -> child occupancy;
 // then per level l = 2..L one or two launches for the lists.
 // The host synchronises once at the end, and also: in cluster-size mode after
-// the sort (to learn each set's depth) and after the full-key sort of the sets
+// the sort (to learn each set's depth) and after each deeper sort of the sets
 // that need one; when the list capacity bound is too large, after the boxes.
 // In graph mode (fmm_set_graphs) the launches of a fixed-depth build up to its
 // first host synchronisation are captured into a CUDA graph, which updates
@@ -460,6 +460,15 @@ int dense_sort_level(uint32_t n, uint32_t peak) {
   return std::min(kMaxLevel, std::max(lvl, 8 * passes_for(lvl) / 3));
 }
 
+// ... and for a cluster-size set whose fullest box at its sort depth Ls holds more
+// than s points (step 1), 8 s (step 2) or 64 s (step 3): were it spread evenly, it
+// would need `step` levels more.  One more than that, for clumps, then as deep as
+// the passes allow.
+int deeper_level(int Ls, int step) {
+  const int lvl = Ls + step + 1;
+  return std::min(kMaxLevel, std::max(lvl, 8 * passes_for(lvl) / 3));
+}
+
 uint64_t wait_ns_of(const fmm_params& p) {
   return (uint64_t)(p.wait_ms ? p.wait_ms : 2000u) * 1000000ull;
 }
@@ -865,7 +874,7 @@ int depth_sets(fmm_ctx* c, std::vector<SetPlan*>& sets, const SortMem& m, uint32
                  c->st, s);
   }
   const size_t need = 64 + sizeof(uint32_t) * nsets;
-  FMM_TRY(build_sync(c));  // the read-back buffer may be replaced
+  if (need > c->rb_bytes) FMM_TRY(build_sync(c));  // the read-back buffer is replaced
   FMM_TRY(pinned_reserve(&c->rb_buf, &c->rb_bytes, need));
   char* h = static_cast<char*>(c->rb_buf);
   FMM_CUDA(cudaMemcpyAsync(h, c->st, sizeof(DevStatus), cudaMemcpyDeviceToHost, s));
@@ -1649,27 +1658,41 @@ int do_builds_on(fmm_ctx* c, const PairIn* pairs, uint32_t npairs, const fmm_par
     }
     if (any_smode) {
       // Cluster-size mode (Sec. 2.1): the deepest level at which s + 1 sorted
-      // points still share a box, per set; sets whose boxes are still too
-      // full at the sort depth are sorted on all key bits and measured again.
-      std::vector<SetPlan*> ss;
-      for (uint32_t i = 0; i < sets.size(); ++i)
-        if (in_smode[i]) ss.push_back(&sets[i]);
+      // points still share a box, per set.
       // (measured over all sorted sets: the sort's descriptors are in that order)
       DevStatus st{};
       FMM_TRY(depth_sets(c, lsd, sm, prm.s, &st));
       if (st.code) return (int)st.code;
-      // A set still too full at its sort depth is sorted three levels deeper
-      // (one or two more radix passes) and measured again; only if that is not
-      // deep enough either, on all key bits.
+      // A set still too full at its sort depth is sorted deeper and measured again;
+      // only if that is not deep enough either, on all key bits.  The other set of
+      // its job needs its order to the same depth, and is sorted along with it: the
+      // passes of such sets are launches more than work (10^6 clumped points and a
+      // partner: 12 radix passes and 640 us with a sort of its own later, 7 and 572).
       for (int round = 0; round < 2; ++round) {
         std::vector<SetPlan*> deep;
-        for (auto* sp : ss)
-          if (!sp->full && sp->depth > (uint32_t)sp->Ls) {
-            if (round == 0 && sp->Ls + 3 < kMaxLevel)
-              sp->Ls += 3;
-            else
-              sp->full = true;
-            deep.push_back(sp);
+        std::vector<int> along(sets.size(), 0);  // depth that a set's partner is sorted to
+        std::vector<uint8_t> is_deep(sets.size(), 0);
+        for (uint32_t i = 0; i < sets.size(); ++i) {
+          SetPlan& sp = sets[i];
+          if (!in_smode[i] || sp.full || sp.depth <= (uint32_t)sp.Ls) continue;
+          is_deep[i] = 1;
+          const int lvl = deeper_level(sp.Ls, (int)sp.depth - sp.Ls);
+          if (round == 0 && lvl < kMaxLevel) {
+            for (const auto& jp : jobs)
+              if (jp.L < 0 && (jp.src == i || jp.recv == i)) {
+                int& other = along[jp.src == i ? jp.recv : jp.src];
+                other = std::max(other, lvl);
+              }
+            sp.Ls = lvl;
+          } else {
+            sp.full = true;
+          }
+          deep.push_back(&sp);
+        }
+        for (uint32_t i = 0; i < sets.size(); ++i)
+          if (!box_order && !is_deep[i] && !sets[i].full && along[i] > sets[i].Ls) {
+            sets[i].Ls = along[i];
+            deep.push_back(&sets[i]);
           }
         if (deep.empty()) break;
         SortMem sd;

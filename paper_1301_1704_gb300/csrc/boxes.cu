@@ -568,7 +568,9 @@ uint32_t occupancy_units(uint32_t n) { return 1u + n / 16384u; }
 // the level-l prefix.  One pass over the pairs (i, i + s) therefore gives,
 // for every set, D = max_i (deepest level shared by points i and i + s),
 // capped at Ls; written as D + 1 by atomicMax into out[set] (zeroed, so 0
-// means "no pair": the set has at most s points).  Units are sort tiles.
+// means "no pair": the set has at most s points).  A set whose level-Ls boxes
+// are too full gets Ls + 1, + 2 or + 3 for a box of more than s, 8 s or 64 s
+// points: how much deeper it is worth sorting.  Units are sort tiles.
 __global__ void __launch_bounds__(256) depth_kernel(const Seg* __restrict__ segs,
                                                     const Slot* __restrict__ slots,
                                                     uint32_t nslots, uint32_t s,
@@ -584,10 +586,21 @@ __global__ void __launch_bounds__(256) depth_kernel(const Seg* __restrict__ segs
   const uint64_t* keys = sg.skeys;
   const uint32_t cap = (uint32_t)sg.Ls;
   uint32_t m = 0;
+  uint64_t too_full = 0;
   for (uint64_t i = t0 + threadIdx.x; i < t0 + sg.tile && i < npairs; i += blockDim.x) {
     const uint32_t shared = first_diff_level(keys[i], keys[i + s]) - 1u;  // 0..21
     const uint32_t v = (shared < cap ? shared : cap) + 1u;
     m = v > m ? v : m;
+    if (v > cap) too_full = i;
+  }
+  // One point of a too full level-Ls box a thread: more than 8 s, 64 s points?  (Only
+  // how deep to sort next: for every point it took a third of the kernel's time.)
+  if (m > cap && too_full + 8ull * s < sg.n) {
+    const uint64_t key = keys[too_full];
+    if (first_diff_level(key, keys[too_full + 8ull * s]) > cap) {
+      ++m;
+      if (too_full + 64ull * s < sg.n && first_diff_level(key, keys[too_full + 64ull * s]) > cap) ++m;
+    }
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
