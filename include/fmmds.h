@@ -287,7 +287,7 @@ int fmm_last_launch_count(fmm_ctx* ctx, uint64_t* launches);
  * CUDA graph, which updates the executable graph kept from the previous build
  * (or replaces it when the work changed shape) and is launched.  A
  * time-stepping caller that rebuilds from the same device buffers with new
- * coordinates launches one graph per build instead of some thirty kernels.
+ * coordinates launches one graph per build instead of some fifteen kernels.
  * Results are identical to the eager build.  Cluster-size builds, builds with
  * per-kernel timing, with FMM_FLAG_HOST_INPUT or with the stall test flag run
  * eagerly.  Disabling frees the kept graph.  Errors: FMM_ERR_ARG for a null
