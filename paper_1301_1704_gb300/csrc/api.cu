@@ -1665,34 +1665,32 @@ int do_builds_on(fmm_ctx* c, const PairIn* pairs, uint32_t npairs, const fmm_par
       if (st.code) return (int)st.code;
       // A set still too full at its sort depth is sorted deeper and measured again;
       // only if that is not deep enough either, on all key bits.  The other set of
-      // its job needs its order to the same depth, and is sorted along with it: the
-      // passes of such sets are launches more than work (10^6 clumped points and a
-      // partner: 12 radix passes and 640 us with a sort of its own later, 7 and 572).
+      // its job needs its order to one level more than this set's at least, and where
+      // it is not sorted to that it is sorted along: the passes of such sets are
+      // launches more than work (10^6 clumped points and a partner: 12 radix passes
+      // and 640 us with a sort of its own later, 7 and 572).
       for (int round = 0; round < 2; ++round) {
         std::vector<SetPlan*> deep;
-        std::vector<int> along(sets.size(), 0);  // depth that a set's partner is sorted to
-        std::vector<uint8_t> is_deep(sets.size(), 0);
+        std::vector<int> least(sets.size(), 0);  // depth that a too full set's job needs
         for (uint32_t i = 0; i < sets.size(); ++i) {
           SetPlan& sp = sets[i];
           if (!in_smode[i] || sp.full || sp.depth <= (uint32_t)sp.Ls) continue;
-          is_deep[i] = 1;
           const int lvl = deeper_level(sp.Ls, (int)sp.depth - sp.Ls);
           if (round == 0 && lvl < kMaxLevel) {
-            for (const auto& jp : jobs)
-              if (jp.L < 0 && (jp.src == i || jp.recv == i)) {
-                int& other = along[jp.src == i ? jp.recv : jp.src];
-                other = std::max(other, lvl);
-              }
+            least[i] = sp.Ls + 1;
             sp.Ls = lvl;
           } else {
             sp.full = true;
           }
           deep.push_back(&sp);
         }
-        for (uint32_t i = 0; i < sets.size(); ++i)
-          if (!box_order && !is_deep[i] && !sets[i].full && along[i] > sets[i].Ls) {
-            sets[i].Ls = along[i];
-            deep.push_back(&sets[i]);
+        for (const auto& jp : jobs)
+          for (int k = 0; k < 2; ++k) {
+            const uint32_t i = k ? jp.src : jp.recv, other = k ? jp.recv : jp.src;
+            SetPlan& sp = sets[other];
+            if (jp.L >= 0 || box_order || least[i] <= sp.Ls || sp.full) continue;
+            if (std::find(deep.begin(), deep.end(), &sp) == deep.end()) deep.push_back(&sp);
+            sp.Ls = sets[i].Ls;
           }
         if (deep.empty()) break;
         SortMem sd;
