@@ -82,7 +82,12 @@ __global__ void __launch_bounds__(kBkPlanThreads) bucket_plan_kernel(const BkSet
   __shared__ uint64_t s_w[W];
   __shared__ uint32_t s_max[W];
   grid_wait(bsets);
-  if (failed(st)) return;
+  // An error of an earlier kernel: the build is over.  One thread decides for the
+  // block, and a set too full for its blocks does not count: another block may
+  // record one while this one starts, and every such set leaves its fullest
+  // sub-cell here.
+  const uint32_t code = threadIdx.x == 0 ? ld_relaxed_u32(&st->code) : 0u;
+  if (__syncthreads_or(code != 0 && code != kStatusBucketFull)) return;
   const BkSet& S = bsets[blockIdx.x];
   const uint32_t cells = bk_cells(S.bl);
   const uint32_t per = (cells + kBkPlanThreads - 1) / kBkPlanThreads;
