@@ -194,7 +194,6 @@ __global__ void __launch_bounds__(kScThreads, 1) bucket_scatter_kernel(
     uint32_t t_first, DevStatus* st) {
   extern __shared__ uint32_t s_at[];  // per sub-cell: the tile's count, then its next slot
   grid_wait(bsets, slots);
-  if (failed(st)) return;
   const uint32_t unit = blockIdx.x + t_first;  // (a launch may start past unit 0)
   const Slot sl = slots[find_slot(slots, nslots, unit)];
   const BkSet& S = bsets[sl.seg];
@@ -204,8 +203,10 @@ __global__ void __launch_bounds__(kScThreads, 1) bucket_scatter_kernel(
   const int sh = 63 - 3 * bl1, lsh = 1 + 3 * bl1;
   const uint64_t keep1 = S.keep << 3;
   for (uint32_t c = threadIdx.x; c < subs; c += blockDim.x) s_at[c] = 0;
-  // a sub-cell of the set is known to be too full: the build will be redone
-  if (__syncthreads_or(threadIdx.x == 0 && ld_relaxed_u32(S.info + 2) != 0)) return;
+  // The build failed, or a sub-cell of the set is known to be too full and the build
+  // will be redone.  One thread decides for the block: other blocks of this launch
+  // record points outside the cube and full sub-cells meanwhile.
+  if (__syncthreads_or(threadIdx.x == 0 && (failed(st) || ld_relaxed_u32(S.info + 2) != 0))) return;
   const uint64_t base = (uint64_t)t * S.tile;
   const uint32_t cnt = (uint32_t)((S.n - base) < (uint64_t)S.tile ? (S.n - base) : S.tile);
   const float* xyz = S.xyz + 3 * base;
