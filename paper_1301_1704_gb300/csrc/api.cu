@@ -1629,6 +1629,39 @@ int do_builds_on(fmm_ctx* c, const PairIn* pairs, uint32_t npairs, const fmm_par
     if (!sp.bucket) lsd.push_back(&sp);
   BucketMem bm;
   FMM_TRY(bucket_setup(c, sets, &bm));
+  // A bucket too full for one block (status kStatusBucketFull, recorded by the
+  // plan and first read back after the boxes or, in a build that also has
+  // cluster-size jobs, with their depths): the build stopped there; build again
+  // with those sets on the radix path.
+  const auto rebuild_full = [&]() -> int {
+    if (c->no_bucket.size() < sets.size()) c->no_bucket.resize(sets.size(), 0);
+    std::vector<uint32_t> info(4 * (size_t)bm.count(), 0);
+    for (uint32_t k = 0; k < bm.count(); ++k)
+      FMM_CUDA(cudaMemcpyAsync(&info[4 * k], bm.host[k].info, sizeof(uint32_t) * 4,
+                               cudaMemcpyDeviceToHost, s));
+    FMM_CUDA(cudaStreamSynchronize(s));
+    bool any = false;
+    for (uint32_t k = 0; k < bm.count(); ++k) {
+      const uint32_t i = bm.host[k].seg;
+      if (!info[4 * k + 2]) continue;
+      any = true;
+      const uint32_t peak = std::max<uint32_t>(info[4 * k + 1], kBkCap + 1);
+      c->no_bucket[i] = peak;
+      auto f = std::find_if(c->full_sets.begin(), c->full_sets.end(), [&](const fmm_ctx::FullSet& x) {
+        return x.xyz == sets[i].orig && x.n == sets[i].n;
+      });
+      if (f != c->full_sets.end()) {
+        f->peak = peak;
+      } else {
+        if (c->full_sets.size() >= 1024) c->full_sets.erase(c->full_sets.begin());
+        c->full_sets.push_back({sets[i].orig, sets[i].n, peak});
+      }
+    }
+    if (!any) return FMM_ERR_CUDA;  // (cannot happen: the status comes with the word)
+    cap_abort(c);
+    c->graph_build = false;
+    return do_builds_on(c, pairs, npairs, prm, outs);
+  };
   // A pipelined build whose sets all take the bucket path also boxes each
   // set as soon as it is sorted (inside run_build, once the outputs exist),
   // so that the sources' box stage runs under the receivers' copy too.
@@ -1662,6 +1695,7 @@ int do_builds_on(fmm_ctx* c, const PairIn* pairs, uint32_t npairs, const fmm_par
       // (measured over all sorted sets: the sort's descriptors are in that order)
       DevStatus st{};
       FMM_TRY(depth_sets(c, lsd, sm, prm.s, &st));
+      if (st.code == kStatusBucketFull) return rebuild_full();
       if (st.code) return (int)st.code;
       // A set still too full at its sort depth is sorted deeper and measured again;
       // only if that is not deep enough either, on all key bits.  The other set of
@@ -1766,37 +1800,7 @@ int do_builds_on(fmm_ctx* c, const PairIn* pairs, uint32_t npairs, const fmm_par
     return FMM_OK;
   };
   const int rs = run_build(c, sets, jobs, prm, bm, &rb, early_boxes ? &copy_sort_box : nullptr);
-  // A bucket too full for one block (status kStatusBucketFull): the build
-  // stopped there; build again with those sets on the radix path.
-  if (rs == (int)kStatusBucketFull) {
-    if (c->no_bucket.size() < sets.size()) c->no_bucket.resize(sets.size(), 0);
-    std::vector<uint32_t> info(4 * (size_t)bm.count(), 0);
-    for (uint32_t k = 0; k < bm.count(); ++k)
-      FMM_CUDA(cudaMemcpyAsync(&info[4 * k], bm.host[k].info, sizeof(uint32_t) * 4,
-                               cudaMemcpyDeviceToHost, s));
-    FMM_CUDA(cudaStreamSynchronize(s));
-    bool any = false;
-    for (uint32_t k = 0; k < bm.count(); ++k) {
-      const uint32_t i = bm.host[k].seg;
-      if (!info[4 * k + 2] && !(rb.seg_long[i] & 2u)) continue;
-      any = true;
-      const uint32_t peak = std::max<uint32_t>(info[4 * k + 1], kBkCap + 1);
-      c->no_bucket[i] = peak;
-      auto f = std::find_if(c->full_sets.begin(), c->full_sets.end(), [&](const fmm_ctx::FullSet& x) {
-        return x.xyz == sets[i].orig && x.n == sets[i].n;
-      });
-      if (f != c->full_sets.end()) {
-        f->peak = peak;
-      } else {
-        if (c->full_sets.size() >= 1024) c->full_sets.erase(c->full_sets.begin());
-        c->full_sets.push_back({sets[i].orig, sets[i].n, peak});
-      }
-    }
-    if (!any) return FMM_ERR_CUDA;  // (cannot happen: the status comes with the bit)
-    cap_abort(c);
-    c->graph_build = false;
-    return do_builds_on(c, pairs, npairs, prm, outs);
-  }
+  if (rs == (int)kStatusBucketFull) return rebuild_full();
   FMM_TRY(rs);
   // Boxes that outran the finishing window, or runs of points tied in an
   // item's key bits too long for one thread (bit 1): redo those orders in
