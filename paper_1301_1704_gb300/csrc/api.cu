@@ -633,10 +633,12 @@ SortTables plan_sort(const std::vector<SetPlan*>& sets) {
 int run_sort(fmm_ctx* c, std::vector<SetPlan*>& sets, SortMem& m, bool stall, uint64_t wait_ns) {
   cudaStream_t s = c->stream;
   int err = FMM_OK;
-  bool any_full = false;  // a set sorted in full (or exactly) keeps every pass stable
+  // A set sorted in full (on all key bits, which is every sort to level 21) or
+  // exactly keeps every pass stable: no finishing sort puts its ties in order.
+  bool any_full = false;
   bool any_exact = false;
   for (auto* sp : sets) {
-    any_full |= sp->full || sp->exact;
+    any_full |= sp->Ls >= kMaxLevel || sp->exact;
     any_exact |= sp->exact;
   }
   const bool onesweep = stall || (c->tuning.sort_kind == FMM_SORT_ONESWEEP && !any_exact);
