@@ -51,23 +51,24 @@ __global__ void __launch_bounds__(256) child_sides_kernel(const uint32_t* __rest
 
 // Whether any of the list entries idx[a..b) has its byte of `side` pass `hit`,
 // for the box of an eight-lane group (uniform over the group); the whole warp
-// calls.
+// calls.  (Counted from the row's first entry: a level's entries may end at 2^32 - 1.)
 template <class Hit>
 __device__ __forceinline__ bool any_entry(const uint32_t* __restrict__ idx, uint32_t a, uint32_t b,
                                           const uint8_t* __restrict__ side, const Hit& hit) {
   const uint32_t lane = threadIdx.x & 31u, l8 = lane & 7u, group = 0xffu << (lane & 24u);
+  const uint32_t* const row = idx + a;
+  const uint32_t n = b - a;  // at most 189
   bool found = false;
-  while (__any_sync(0xffffffffu, !found && a < b)) {
+  for (uint32_t i = 0; __any_sync(0xffffffffu, !found && i < n); i += 32) {
     bool h = false;
     if (!found) {
 #pragma unroll
       for (int u = 0; u < 4; ++u) {  // the loads of 32 entries together
-        const uint32_t j = a + l8 + 8u * u;
-        if (j < b) h |= hit(side[idx[j]]);
+        const uint32_t j = i + l8 + 8u * u;
+        if (j < n) h |= hit(side[row[j]]);
       }
     }
     found |= (__ballot_sync(0xffffffffu, h) & group) != 0;
-    a += 32;
   }
   return found;
 }
