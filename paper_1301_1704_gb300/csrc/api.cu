@@ -1805,8 +1805,7 @@ int do_builds_on(fmm_ctx* c, const PairIn* pairs, uint32_t npairs, const fmm_par
   if (rs == (int)kStatusBucketFull) return rebuild_full();
   FMM_TRY(rs);
   // Boxes that outran the finishing window, or runs of points tied in an
-  // item's key bits too long for one thread (bit 1): redo those orders in
-  // full.
+  // item's key bits too long for one thread: redo those orders in full.
   std::vector<uint32_t> longs;
   for (uint32_t i = 0; i < sets.size(); ++i)
     if (rb.seg_long[i]) longs.push_back(i);

@@ -179,8 +179,8 @@ __global__ void __launch_bounds__(kBkPlanThreads) bucket_plan_kernel(const BkSet
 // point).  Sub-cell c's items occupy slots [c kBkCap, c kBkCap + count): the
 // totals are not known while the tiles run, so every sub-cell has room for
 // the most points one block sorts; a fuller sub-cell keeps only what fits
-// (the boxes stage then stops the build and the host redoes the set by the
-// radix path).  The order inside a sub-cell is left to the atomics: the
+// (the plan then stops the build and the host redoes the set by the radix
+// path).  The order inside a sub-cell is left to the atomics: the
 // boxes stage orders each sub-cell by whole item.  The stores of a warp land
 // in many sub-cells, each a part of a 32-byte sector that the tile and its
 // neighbours in tile order fill over time; one block an SM (few tiles in
@@ -431,21 +431,7 @@ __global__ void __launch_bounds__(kBkThreads, 3) bucket_boxes_kernel(
   const uint64_t imask = (1ull << ib) - 1ull, keep1 = S.keep;
   const uint32_t nsub = S.nsub, u = S.u, d0 = S.d0;
   uint64_t* const status = S.status;  // [kLevels][nsub]: one chain of sub-cells per level
-  const uint32_t n_j = S.n, offj = S.off, cell1 = S.key;
-  if (n_j > (uint32_t)kBkCap) {
-    // More points than a block sorts: the host builds this set again by the
-    // radix path.  The build stops here (later kernels see the status and
-    // leave their outputs alone); empty counts are published so that later
-    // sub-cells do not wait.
-    if (tid == 0) {
-      atomicOr(G.seg_long, 2u);
-      atomicExch(&st->seg_long, 1u);
-      set_error(st, kStatusBucketFull);
-    }
-    for (int l = tid; l <= Lb; l += kBkThreads)
-      st_relaxed(status + (uint64_t)l * nsub + u, u == 0 ? kFlagIncl : kFlagAgg);
-    return;
-  }
+  const uint32_t n_j = S.n, offj = S.off, cell1 = S.key;  // n_j <= kBkCap: the plan passed it
 
   // The output level arrays, read once (their loads overlap the items').
   if (tid <= Lb) {

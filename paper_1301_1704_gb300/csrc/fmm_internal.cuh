@@ -46,7 +46,7 @@ __device__ __forceinline__ uint64_t global_timer_ns() {
 // ---------------------------------------------------------------------------
 // Morton code.  Ten bits at a time are spread three apart with the usual
 // shift-and-mask ladder (each step halves the width of the bit groups still to be
-// spread: 8 -> 4 -> 2 -> 1 bits) in 32-bit words; compact3 undoes it.
+// spread: 8 -> 4 -> 2 -> 1 bits) in 32-bit words.
 __device__ __forceinline__ uint32_t spread10(uint32_t v) {  // v < 2^10
   v = (v | (v << 16)) & 0x030000ffu;
   v = (v | (v << 8)) & 0x0300f00fu;
@@ -66,16 +66,6 @@ __device__ __forceinline__ uint64_t interleave21(uint32_t x, uint32_t y, uint32_
   const uint32_t mid = interleave10((x >> 1) & 0x3ffu, (y >> 1) & 0x3ffu, (z >> 1) & 0x3ffu);
   const uint32_t lo = (x & 1u) + 2u * (y & 1u) + 4u * (z & 1u);
   return ((uint64_t)hi << 33) | ((uint64_t)mid << 3) | lo;
-}
-
-__device__ __forceinline__ uint32_t compact3(uint64_t x) {
-  x &= 0x1249249249249249ull;
-  x = (x ^ (x >> 2)) & 0x10c30c30c30c30c3ull;
-  x = (x ^ (x >> 4)) & 0x100f00f00f00f00full;
-  x = (x ^ (x >> 8)) & 0x001f0000ff0000ffull;
-  x = (x ^ (x >> 16)) & 0x001f00000000ffffull;
-  x = (x ^ (x >> 32)) & 0x1fffffull;
-  return (uint32_t)x;
 }
 
 // Cell of one coordinate at level 21; false if outside [0, 1] or NaN.
@@ -243,22 +233,6 @@ __device__ __forceinline__ uint64_t lookback_warp(const uint64_t* status, uint32
     if (upto == 0 && clk.expired(st, wait_ns)) break;
   }
   return excl;
-}
-
-// Store v when `word` is non-zero, as one predicated instruction (streaming
-// cache hint): no branch around it.
-__device__ __forceinline__ void st_cs_if(uint32_t* p, uint32_t v, uint32_t word) {
-  asm volatile(
-      "{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\t@q st.global.cs.u32 [%0], %1;\n\t}"
-      ::"l"(p), "r"(v), "r"(word)
-      : "memory");
-}
-// ... and when `word` is zero.
-__device__ __forceinline__ void st_cs_if_zero(uint32_t* p, uint32_t v, uint32_t word) {
-  asm volatile(
-      "{\n\t.reg .pred q;\n\tsetp.eq.u32 q, %2, 0;\n\t@q st.global.cs.u32 [%0], %1;\n\t}"
-      ::"l"(p), "r"(v), "r"(word)
-      : "memory");
 }
 
 // ---------------------------------------------------------------------------
