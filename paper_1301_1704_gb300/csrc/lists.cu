@@ -709,6 +709,7 @@ __global__ void __launch_bounds__(kListThreads, 4) list_fill_kernel(
   for (uint32_t u = blockIdx.x * kFillWarps + warp; u < chunks * split; u += warps) {
     const uint32_t c = u / split;  // (a power of two)
     if (c >= jend) {  // c only grows
+      __syncwarp();   // every lane has read the last job
       if (lane == 0) {
         load_job(W, segs, jobs, njobs, l, LV, up, one, np1, c);
         W.base2 = njobs == 1 ? 0ull : LV.jbase[2 * W.j];
