@@ -37,7 +37,9 @@ __device__ __forceinline__ uint32_t first_diff_level(uint64_t a, uint64_t b) {
   return x == 0 ? 22u : (uint32_t)((2 + __clzll((long long)x)) / 3);
 }
 
-__global__ void __launch_bounds__(kBoxThreads) finish_boxes_kernel(const Seg* __restrict__ segs,
+// (Four blocks an SM, which shared memory allows: with three, 512 sets of 7.4e7 points
+// take 788 us for 737.)
+__global__ void __launch_bounds__(kBoxThreads, 4) finish_boxes_kernel(const Seg* __restrict__ segs,
                                                                    const Slot* __restrict__ slots,
                                                                    uint32_t nslots, DevStatus* st,
                                                                    uint64_t wait_ns) {
@@ -154,17 +156,27 @@ __global__ void __launch_bounds__(kBoxThreads) finish_boxes_kernel(const Seg* __
     const int lowbits = 63 - 3 * Ls;
     const uint64_t lowmask = lowbits >= 64 ? ~0ull : ((1ull << lowbits) - 1ull);
     // The points of a box differ in their low key bits only: the top 32 of those
-    // take the keys' low words (the boxes' keys below need the high words alone,
-    // to depth 10), and points are compared by them; points that agree there
-    // too, by the keys the sort left.  A box is compared all against all, so these
+    // take the keys' low words, and points are compared by them.  The bits they push
+    // out take the place that they leave in the high words, below the box's prefix,
+    // so that points that agree in the low words are ordered by the high ones, then by
+    // index.  (The boxes' keys below need the prefix alone, Lb <= Ls; past level 10
+    // the prefix reaches the low words.)  A box is compared all against all, so these
     // loads and compares are most of the kernel's instructions: 7.4e7 points in 512
-    // sets 882 -> 740 us, 2 x 2^24 points on a sphere and in clumps 356 -> 309.
+    // sets 882 -> 737 us, 2 x 2^24 points on a sphere and in clumps 356 -> 307; 8192
+    // points 250 times over 539 -> 627 (1014 with the tied points' keys from memory).
     const bool words = Lb <= 10;
-    uint32_t* const low = reinterpret_cast<uint32_t*>(sk + 1);  // low[2 j]: point j
+    uint2* const word = reinterpret_cast<uint2*>(sk + 1);  // point j: x low, y high
     if (words) {
+      const int over = lowbits - 32;  // bits pushed out
       for (int j = threadIdx.x; j < jend; j += kBoxThreads) {
-        const uint64_t k = sk[j + 1] & lowmask;
-        low[2 * j] = (uint32_t)(lowbits > 32 ? k >> (lowbits - 32) : k);
+        const uint64_t k = sk[j + 1];
+        uint32_t lo = (uint32_t)(k & lowmask), hi = (uint32_t)(k >> 32);
+        if (over > 0) {
+          const uint32_t out = (1u << over) - 1u;
+          hi = (hi & ~out) | (lo & out);
+          lo = (uint32_t)(k >> over);
+        }
+        word[j] = make_uint2(lo, hi);
       }
       __syncthreads();
     }
@@ -199,19 +211,18 @@ __global__ void __launch_bounds__(kBoxThreads) finish_boxes_kernel(const Seg* __
       }
       uint32_t r = 0;
       if (words && b - a > 1) {
-        const uint32_t mine = low[2 * j];
+        const uint32_t mine = word[j].x;
         uint32_t alike = 0;
         for (int q = a; q < b; ++q) {
-          const uint32_t k = low[2 * q];
+          const uint32_t k = word[q].x;
           r += k < mine;
           alike += k == mine;
         }
         if (alike > 1) {  // more than the point itself
-          const uint64_t key = keys[t0 + j];
+          const uint32_t hj = word[j].y, vj = s_val[j];
           for (int q = a; q < b; ++q) {
-            if (low[2 * q] != mine || q == j) continue;
-            const uint64_t kq = keys[t0 + q];
-            r += kq < key || (kq == key && s_val[q] < s_val[j]);
+            const uint2 k = word[q];
+            r += k.x == mine && (k.y < hj || (k.y == hj && s_val[q] < vj));
           }
         }
       } else if (b - a > 1) {
