@@ -1824,9 +1824,9 @@ int do_builds_on(fmm_ctx* c, const PairIn* pairs, uint32_t npairs, const fmm_par
 // A build, in graph mode when the context asks for it: a fixed-depth build
 // (no cluster-size job), from the second build of a context on (the first
 // one grows the arena and the staging buffers), and not with timing, the
-// stall test or copies from the caller's host memory.  Its launches up to the
-// first host synchronisation -- the whole build but the read-back, unless
-// the list capacity is too large to reserve up front -- are one graph.
+// stall test or copies from the caller's host memory.  Its work up to the
+// first host synchronisation -- the whole build with its read-back, unless
+// the list capacity is too large to reserve up front -- is one graph.
 int do_builds(fmm_ctx* c, const PairIn* pairs, uint32_t npairs, const fmm_params& prm,
               fmm_tree* outs) {
   const uint32_t f = prm.flags;

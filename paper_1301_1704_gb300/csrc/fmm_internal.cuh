@@ -606,11 +606,10 @@ void launch_list_fill(const Seg* segs, const Job* jobs, uint32_t njobs, int l,
                       const ListLevel& lv, const ListLevel& up, const LevelJob& one,
                       uint32_t max_chunks, DevStatus* st, cudaStream_t s);
 
-// Bucket path (bucket.cu).  count and scatter: units = tiles of the slots'
-// sets (slot seg = BkSet index); plan: one block per set; split: units =
-// bucket slots (slot unit0 = the set's first bucket slot); boxes: units =
-// bucket slots as for split, 8 blocks each (one per sub-cell), taken in
-// order by ticket (slot unit0 = the set's first sub-cell slot).
+// Bucket path (bucket.cu).  scatter: units = tiles of the slots' sets (slot
+// seg = BkSet index); plan: one block per set; boxes: units = bucket slots,
+// 8 blocks each (one per sub-cell), taken in order by ticket (slot unit0 = the
+// set's first sub-cell slot).
 void launch_bucket_plan(const BkSet* bsets, uint32_t nsets, DevStatus* st, cudaStream_t s);
 // Tiles [t_first, t_first + tiles) of the launch's units.
 void launch_bucket_scatter(const BkSet* bsets, const Slot* slots, uint32_t nslots, uint32_t t_first,
